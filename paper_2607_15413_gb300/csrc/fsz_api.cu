@@ -126,7 +126,7 @@ fsz_status prepare_one(const float* d_in, fsz_dims dims, fsz_eb_mode mode, doubl
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const KernelArgs a = make_args(d_ws, call.L);
   launch_setup_compress(a, call.desc, call.L.chunk_cap, s);  // (clears the workspace it uses)
-  if (call.desc.nchunks > 0) launch_stats(a, s);
+  if (call.desc.nchunks > 0) launch_stats(a, s, true);
   return launched();
 }
 
@@ -284,7 +284,7 @@ fsz_status fsz_compress_batched(const fsz_cfield* d_fields, uint32_t nfields, ui
   if (cudaMemsetAsync(d_ws, 0, L.bytes, s) != cudaSuccess) return FSZ_ERR_CUDA;
   const KernelArgs a = make_args(d_ws, L);
   launch_plan_compress(a, d_fields, nfields, L.chunk_cap, s);
-  launch_stats(a, s);
+  launch_stats(a, s, false);
   launch_compress(a, s, kCompressFeatures);  // fields may switch features off
   return launched();
 }

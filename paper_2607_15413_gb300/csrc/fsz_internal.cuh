@@ -565,7 +565,7 @@ LaunchCfg stats_cfg();
 LaunchCfg compress_cfg();
 LaunchCfg decompress_cfg();
 
-void launch_stats(const KernelArgs& a, cudaStream_t st);
+void launch_stats(const KernelArgs& a, cudaStream_t st, bool single);
 // Compression kernel instances (feature-toggle builds of one kernel): the full method;
 // with switched-off features honoured per field (fsz_compress_features, batches); the
 // multipass evaluation's encoding pass (selection from a.given_costs).

@@ -107,7 +107,7 @@ extern "C" fsz_status fsz_compress_noalloc(const float* d_in, fsz_dims dims, fsz
   a.timeout_ns = kDefaultTimeoutNs;
   launch_setup_compress(a, desc, L.chunk_cap, s);
   if (desc.nchunks > 0) {
-    launch_stats(a, s);
+    launch_stats(a, s, true);
     launch_compress(a, s);
   }
   if (d_status != nullptr &&
