@@ -126,7 +126,7 @@ fsz_status prepare_one(const float* d_in, fsz_dims dims, fsz_eb_mode mode, doubl
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const KernelArgs a = make_args(d_ws, call.L);
   launch_setup_compress(a, call.desc, call.L.chunk_cap, s);  // (clears the workspace it uses)
-  if (call.desc.nchunks > 0) launch_stats(a, s, true);
+  if (call.desc.nchunks > 0) launch_stats(a, d_in, call.desc.n, s);
   return launched();
 }
 
@@ -143,7 +143,7 @@ fsz_status decompress_one(const void* d_in, uint64_t in_bytes, float* d_out,
   const KernelArgs a = make_args(d_ws, L);
   launch_setup_decompress(a, static_cast<const uint8_t*>(d_in), in_bytes, d_out, out_capacity_elems,
                           L.chunk_cap, s);
-  launch_decompress(a, s, kind);
+  launch_decompress(a, (out_capacity_elems + kDChunkElems - 1) / kDChunkElems, s, kind);
   return launched();
 }
 
@@ -203,7 +203,8 @@ fsz_status fsz_compress_encode(const float* d_in, fsz_dims dims, fsz_eb_mode mod
   fsz_status st = check_compress(d_in, dims, mode, eb, d_out, out_capacity, d_ws, ws_bytes, &call);
   if (st != FSZ_OK) return st;
   if (call.desc.nchunks == 0) return FSZ_OK;
-  launch_compress(make_args(d_ws, call.L), reinterpret_cast<cudaStream_t>(stream), kCompressFull);
+  launch_compress(make_args(d_ws, call.L), call.desc.nchunks, reinterpret_cast<cudaStream_t>(stream),
+                  kCompressFull);
   return launched();
 }
 
@@ -230,7 +231,8 @@ fsz_status fsz_compress_features(const float* d_in, fsz_dims dims, fsz_eb_mode m
   CompressCall call;
   st = check_compress(d_in, dims, mode, eb, d_out, out_capacity, d_ws, ws_bytes, &call, features_off);
   if (st != FSZ_OK || call.desc.nchunks == 0) return st;
-  launch_compress(make_args(d_ws, call.L), reinterpret_cast<cudaStream_t>(stream), kCompressFeatures);
+  launch_compress(make_args(d_ws, call.L), call.desc.nchunks, reinterpret_cast<cudaStream_t>(stream),
+                  kCompressFeatures);
   return launched();
 }
 
@@ -250,7 +252,7 @@ fsz_status fsz_compress_multipass(const float* d_in, fsz_dims dims, fsz_eb_mode 
   for (int v = 0; v < 4; ++v) launch_cost_pass(a, v, d_costs, s);
   a.given_costs = d_costs;
   a.given_T = call.desc.T;
-  launch_compress(a, s, kCompressGiven);
+  launch_compress(a, call.desc.nchunks, s, kCompressGiven);
   return launched();
 }
 
@@ -284,8 +286,9 @@ fsz_status fsz_compress_batched(const fsz_cfield* d_fields, uint32_t nfields, ui
   if (cudaMemsetAsync(d_ws, 0, L.bytes, s) != cudaSuccess) return FSZ_ERR_CUDA;
   const KernelArgs a = make_args(d_ws, L);
   launch_plan_compress(a, d_fields, nfields, L.chunk_cap, s);
-  launch_stats(a, s, false);
-  launch_compress(a, s, kCompressFeatures);  // fields may switch features off
+  const uint64_t max_chunks = n_total / kCChunkElems + nfields;
+  launch_stats_batch(a, max_chunks, s);
+  launch_compress(a, max_chunks, s, kCompressFeatures);  // fields may switch features off
   return launched();
 }
 
@@ -300,7 +303,7 @@ fsz_status fsz_decompress_batched(const fsz_dfield* d_fields, uint32_t nfields,
   if (cudaMemsetAsync(d_ws, 0, L.bytes, s) != cudaSuccess) return FSZ_ERR_CUDA;
   const KernelArgs a = make_args(d_ws, L);
   launch_plan_decompress(a, d_fields, nfields, L.chunk_cap, s);
-  launch_decompress(a, s);
+  launch_decompress(a, n_total_capacity / kDChunkElems + nfields, s);
   return launched();
 }
 

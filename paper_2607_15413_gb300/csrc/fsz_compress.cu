@@ -424,7 +424,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   CompressSmem& S = *reinterpret_cast<CompressSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint64_t total = a.ctrl->total_chunks;
   // mbarrier waits outlast the longest lookback wait, so a lookback that runs out is
   // reported as such rather than as a stalled pipeline.
   const uint64_t wait_ns = 4 * a.timeout_ns;
@@ -441,7 +440,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     for (int w = 0; w < kWarps; ++w) S.ring_tail[w] = 0;
     fence_mbar_init();
   }
+  grid_wait();
   __syncthreads();
+  const uint64_t total = a.ctrl->total_chunks;
 
   if (warp == kHostWarp) {
     // ---------------------------------------------------------------- host
@@ -808,19 +809,19 @@ LaunchCfg compress_cfg() {
   });
 }
 
-void launch_compress(const KernelArgs& args, cudaStream_t st, CompressKind kind) {
+void launch_compress(const KernelArgs& args, uint64_t max_chunks, cudaStream_t st, CompressKind kind) {
   const LaunchCfg c = compress_cfg();
-  const int g = sched_grid(c, kSchedCompress);
+  const int g = sched_grid(c, kSchedCompress, max_chunks);
   KernelArgs a = args;
   a.ticket_chunks = uint32_t(g_schedule.c_ticket_chunks);
   a.ticket_lead = uint32_t(g_schedule.c_ticket_lead);
   a.min_tickets = uint32_t(g_schedule.min_tickets);
   if (kind == kCompressFeatures)
-    fsz_compress_kernel<false, true><<<g, kThreads, c.smem, st>>>(a);
+    launch_dependent(fsz_compress_kernel<false, true>, g, kThreads, c.smem, st, a);
   else if (kind == kCompressGiven)
-    fsz_compress_kernel<true, false><<<g, kThreads, c.smem, st>>>(a);
+    launch_dependent(fsz_compress_kernel<true, false>, g, kThreads, c.smem, st, a);
   else
-    fsz_compress_kernel<false, false><<<g, kThreads, c.smem, st>>>(a);
+    launch_dependent(fsz_compress_kernel<false, false>, g, kThreads, c.smem, st, a);
 }
 
 }  // namespace fsz

@@ -284,9 +284,7 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
   DecompressSmem& S = *reinterpret_cast<DecompressSmem*>(smem_raw);
   constexpr uint32_t FULL = 0xffffffffu;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint64_t total = a.ctrl->total_chunks;
   const uint64_t wait_ns = 4 * a.timeout_ns;
-  const uint32_t group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
   const uint32_t recs = a.records;
 
   if (tid == 0) {
@@ -297,10 +295,13 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
     }
     fence_mbar_init();
   }
+  grid_wait();
   __syncthreads();
 
   if (warp == kHeaderWarp) {
     // ---------------------------------------------------------------- header warp
+    const uint64_t total = a.ctrl->total_chunks;
+    const uint32_t group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
     const bool single = a.ctrl->nfields == 1;
     for (uint32_t seq = 0;; seq += group) {
       // the group's records must be free: their previous chunks decoded
@@ -619,19 +620,20 @@ LaunchCfg decompress_cfg() {
   });
 }
 
-void launch_decompress(const KernelArgs& args, cudaStream_t st, DecompressKind kind) {
+void launch_decompress(const KernelArgs& args, uint64_t max_chunks, cudaStream_t st,
+                       DecompressKind kind) {
   const LaunchCfg c = decompress_cfg();
-  const int g = sched_grid(c, kSchedDecompress);
+  const int g = sched_grid(c, kSchedDecompress, max_chunks);
   KernelArgs a = args;
   a.ticket_chunks = uint32_t(g_schedule.d_ticket_chunks);
   a.records = uint32_t(g_schedule.d_records);
   a.min_tickets = uint32_t(g_schedule.min_tickets);
   if (kind == kDecompressAny)
-    fsz_decompress_kernel<true, false><<<g, kThreads, c.smem, st>>>(a);
+    launch_dependent(fsz_decompress_kernel<true, false>, g, kThreads, c.smem, st, a);
   else if (kind == kDecompressPrezeroed)
-    fsz_decompress_kernel<false, true><<<g, kThreads, c.smem, st>>>(a);
+    launch_dependent(fsz_decompress_kernel<false, true>, g, kThreads, c.smem, st, a);
   else
-    fsz_decompress_kernel<false, false><<<g, kThreads, c.smem, st>>>(a);
+    launch_dependent(fsz_decompress_kernel<false, false>, g, kThreads, c.smem, st, a);
 }
 
 }  // namespace fsz

@@ -95,8 +95,7 @@ extern "C" fsz_status fsz_compress_noalloc(const float* d_in, fsz_dims dims, fsz
   desc.nchunks = (T + kCChunkTiles - 1) / kCChunkTiles;
 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  // The array keeps the previous call's contents: clear the part this call uses.
-  if (cudaMemsetAsync(ws, 0, L.bytes, s) != cudaSuccess) return FSZ_ERR_CUDA;
+  // (the array keeps the previous call's contents: the set-up kernel clears what it uses)
   uint8_t* base = static_cast<uint8_t*>(ws);
   KernelArgs a;
   a.ctrl = reinterpret_cast<Ctrl*>(base);
@@ -107,8 +106,8 @@ extern "C" fsz_status fsz_compress_noalloc(const float* d_in, fsz_dims dims, fsz
   a.timeout_ns = kDefaultTimeoutNs;
   launch_setup_compress(a, desc, L.chunk_cap, s);
   if (desc.nchunks > 0) {
-    launch_stats(a, s, true);
-    launch_compress(a, s);
+    launch_stats(a, d_in, n, s);
+    launch_compress(a, desc.nchunks, s);
   }
   if (d_status != nullptr &&
       cudaMemcpyAsync(d_status, &a.ctrl->status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s) !=

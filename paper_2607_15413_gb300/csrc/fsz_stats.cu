@@ -89,14 +89,14 @@ struct StatsItem {
 };
 
 template <bool kSingle>
-__global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs a) {
+__global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs a, const float* in,
+                                                                       uint64_t n) {
   constexpr int kStatsWarps = kStatsThreads / 32;
   __shared__ StatsItem s_item[kSegChunks];
   __shared__ float s_lo[kSegChunks][kStatsWarps], s_hi[kSegChunks][kStatsWarps];
   __shared__ uint32_t s_abs[kSegChunks][kStatsWarps];
   __shared__ uint32_t s_f[kSegChunks], s_cnt[kSegChunks];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint64_t total = a.ctrl->total_chunks;
 
   float lo = __int_as_float(0x7f800000), hi = __int_as_float(0xff800000);
   uint32_t mabs = 0;
@@ -171,22 +171,24 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
     // One field: a stride over the grid, from the field's end to its start, so that what the
     // pass leaves in L2 is what the compression kernel reads first (121 x 251 x 269 field,
     // whole call: 38.0 us upwards, 36.3 us downwards; 512^3: equal).
-    if (blockIdx.x >= total) return;
+    // The field is read before grid_wait: the set-up kernel before this one does not write it,
+    // and has itself waited for what came before the call.
+    const uint64_t total = (n + kCChunkElems - 1) / kCChunkElems;  // >= gridDim.x
     const uint64_t gn = (total - blockIdx.x + gridDim.x - 1) / gridDim.x;
-    const FieldInfo* fi = a.fields;
-    const float* const in = fi->in;
-    const uint64_t n = fi->n;
     for (uint64_t k = 0; k < gn; ++k) {
       const uint64_t e0 = (total - 1 - (blockIdx.x + k * gridDim.x)) * uint64_t(kCChunkElems);
       chunk(in + e0, uint32_t(min(n - e0, uint64_t(kCChunkElems))));
     }
     deposit(0, 0, uint32_t(gn));
+    grid_wait();
     __syncthreads();
     if (threadIdx.x == 0) publish(0);
   } else {
     // A batch: each CTA takes one contiguous range of its chunks and so meets few fields
     // (a batch of 32 mixed fields of 258 MB in all, whole call: 145.5 us with a stride over
     // the grid, 142.4 us with ranges).
+    grid_wait();
+    const uint64_t total = a.ctrl->total_chunks;
     const uint64_t g0 = total * blockIdx.x / gridDim.x;
     const uint64_t gn = total * (blockIdx.x + 1) / gridDim.x - g0;
     for (uint64_t k0 = 0; k0 < gn; k0 += kSegChunks) {
@@ -325,6 +327,8 @@ static_assert(sizeof(Ctrl) <= 256 && sizeof(Ctrl) % 8 == 0 && sizeof(FieldInfo) 
               "control words and field record clear as 8-byte words");
 
 __device__ __forceinline__ bool setup_clear(const KernelArgs& a, uint64_t nflags) {
+  grid_wait();
+  grid_release();
   const uint64_t t = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t == 0) {
     uint64_t* c = reinterpret_cast<uint64_t*>(a.ctrl);
@@ -386,6 +390,8 @@ __global__ void __launch_bounds__(kPlanThreads) fsz_plan_kernel(KernelArgs a, co
   __shared__ uint64_t s_warp[kPlanThreads / 32];
   __shared__ uint64_t s_carry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  grid_wait();
+  grid_release();
   if (tid == 0) s_carry = 0;
   __syncthreads();
   for (uint32_t base = 0; base < nfields; base += kPlanThreads) {
@@ -477,34 +483,39 @@ LaunchCfg stats_cfg() {
   });
 }
 
-void launch_stats(const KernelArgs& a, cudaStream_t st, bool single) {
-  const int g = sched_grid(stats_cfg(), kSchedStats);
-  if (single)
-    fsz_stats_kernel<true><<<g, kStatsThreads, 0, st>>>(a);
-  else
-    fsz_stats_kernel<false><<<g, kStatsThreads, 0, st>>>(a);
+void launch_stats(const KernelArgs& a, const float* in, uint64_t n, cudaStream_t st) {
+  const uint64_t chunks = (n + kCChunkElems - 1) / kCChunkElems;
+  launch_dependent(fsz_stats_kernel<true>, sched_grid(stats_cfg(), kSchedStats, chunks), kStatsThreads,
+                   0, st, a, in, n);
+}
+
+void launch_stats_batch(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st) {
+  launch_dependent(fsz_stats_kernel<false>, sched_grid(stats_cfg(), kSchedStats, max_chunks),
+                   kStatsThreads, 0, st, a, nullptr, uint64_t(0));
 }
 
 void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t chunk_cap, cudaStream_t st) {
   const uint64_t nflags = kFlagStride * chunk_cap;
-  fsz_setup_compress_kernel<<<setup_grid(nflags), kSetupThreads, 0, st>>>(a, fi, nflags);
+  launch_dependent(fsz_setup_compress_kernel, setup_grid(nflags), kSetupThreads, 0, st, a, fi, nflags);
 }
 
 void launch_setup_decompress(const KernelArgs& a, const uint8_t* in, uint64_t in_bytes, float* out,
                              uint64_t cap_elems, uint64_t chunk_cap, cudaStream_t st) {
   const uint64_t nflags = kFlagStride * chunk_cap;
-  fsz_setup_decompress_kernel<<<setup_grid(nflags), kSetupThreads, 0, st>>>(a, in, in_bytes, out,
-                                                                            cap_elems, chunk_cap, nflags);
+  launch_dependent(fsz_setup_decompress_kernel, setup_grid(nflags), kSetupThreads, 0, st, a, in,
+                   in_bytes, out, cap_elems, chunk_cap, nflags);
 }
 
 void launch_plan_compress(const KernelArgs& a, const fsz_cfield* d_fields, uint32_t nfields,
                           uint64_t chunk_cap, cudaStream_t st) {
-  fsz_plan_kernel<true><<<1, kPlanThreads, 0, st>>>(a, d_fields, nfields, chunk_cap);
+  launch_dependent(fsz_plan_kernel<true>, 1, kPlanThreads, 0, st, a, static_cast<const void*>(d_fields),
+                   nfields, chunk_cap);
 }
 
 void launch_plan_decompress(const KernelArgs& a, const fsz_dfield* d_fields, uint32_t nfields,
                             uint64_t chunk_cap, cudaStream_t st) {
-  fsz_plan_kernel<false><<<1, kPlanThreads, 0, st>>>(a, d_fields, nfields, chunk_cap);
+  launch_dependent(fsz_plan_kernel<false>, 1, kPlanThreads, 0, st, a, static_cast<const void*>(d_fields),
+                   nfields, chunk_cap);
 }
 
 }  // namespace fsz
