@@ -277,8 +277,8 @@ fsz_status fsz_get_schedule_limits(uint32_t* stats_max, uint32_t* compress_max,
 /* The full launch schedule (no counterpart in the paper, which fixes one tile-to-block
  * mapping; none of it changes a stream). The persistent kernels hand out work by atomic
  * tickets; a ticket covers `*_ticket_chunks` consecutive chunks of 32 tiles (1-4), the
- * unit of work a CTA takes, and in each of its chunks after the first the chunk's byte
- * offset follows from the previous one without a lookback (Sec. 4.4). Compression takes
+ * unit of work a CTA takes; in each of its chunks after the first the chunk's byte offset
+ * follows from the previous one (without a lookback in compression, Sec. 4.4). Compression takes
  * tickets up to `compress_ticket_lead` chunks (1-3) ahead of its compute warps;
  * decompression keeps up to `decompress_records` chunks (2 x ticket chunks .. 16) between
  * ticket and decode per CTA. A launch whose chunks would give fewer than
@@ -456,10 +456,12 @@ fsz_status fsz_server_destroy(fsz_server s);
 /* Device-to-device copy on `stream` (for clients without a CUDA binding of their own). */
 fsz_status fsz_copy_device(void* d_dst, const void* d_src, uint64_t bytes, fsz_stream stream);
 
-/* Test hooks for failure detection (not for production use): the chunk whose global
- * index equals skip_chunk publishes no lookback flag, so its successor's bounded wait
- * runs out after timeout_ns and records FSZ_ERR_TIMEOUT; the kernels still finish.
- * skip_chunk = UINT64_MAX disables the hook; timeout_ns = 0 restores the default (2 s). */
+/* Test hooks for failure detection (not for production use): in compression the chunk whose
+ * global index equals skip_chunk publishes no lookback flag, so its successor's bounded
+ * wait runs out after timeout_ns; in decompression its record is not handed to the decoding
+ * warps, so their bounded wait runs out. Either records FSZ_ERR_TIMEOUT, and the kernels
+ * still finish. skip_chunk = UINT64_MAX disables the hook; timeout_ns = 0 restores the
+ * default (2 s). */
 void fsz_set_test_hooks(uint64_t skip_chunk, uint64_t timeout_ns);
 
 /* Library version and build target, e.g. "fsz 1.0 sm_103a". */

@@ -68,6 +68,8 @@ KernelArgs make_args(void* d_ws, const WsLayout& L) {
   a.fields = reinterpret_cast<FieldInfo*>(ws + L.fields_off);
   a.chunk_field = reinterpret_cast<const uint32_t*>(ws + L.map_off);
   a.flags = reinterpret_cast<uint64_t*>(ws + L.flags_off);
+  a.sums = reinterpret_cast<uint32_t*>(a.flags);
+  a.block_sums = a.sums + L.chunk_cap;
   a.skip_chunk = g_skip_chunk;
   a.timeout_ns = g_timeout_ns;
   return a;
@@ -140,9 +142,12 @@ fsz_status decompress_one(const void* d_in, uint64_t in_bytes, float* d_out,
   const WsLayout L = ws_layout((out_capacity_elems + kTile - 1) / kTile, 1);
   if (ws_bytes < L.bytes) return FSZ_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const KernelArgs a = make_args(d_ws, L);
-  launch_setup_decompress(a, static_cast<const uint8_t*>(d_in), in_bytes, d_out, out_capacity_elems,
-                          L.chunk_cap, s);
+  KernelArgs a = make_args(d_ws, L);
+  a.sin = static_cast<const uint8_t*>(d_in);
+  a.in_bytes = in_bytes;
+  a.dout = d_out;
+  a.cap_elems = out_capacity_elems;
+  launch_setup_decompress(a, L.chunk_cap, s);
   launch_decompress(a, (out_capacity_elems + kDChunkElems - 1) / kDChunkElems, s, kind);
   return launched();
 }
@@ -300,10 +305,12 @@ fsz_status fsz_decompress_batched(const fsz_dfield* d_fields, uint32_t nfields,
   const WsLayout L = ws_layout(n_total_capacity / kTile + nfields, nfields);
   if (ws_bytes < L.bytes) return FSZ_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(d_ws, 0, L.bytes, s) != cudaSuccess) return FSZ_ERR_CUDA;
+  if (cudaMemsetAsync(d_ws, 0, L.map_off, s) != cudaSuccess) return FSZ_ERR_CUDA;  // (control, fields)
   const KernelArgs a = make_args(d_ws, L);
   launch_plan_decompress(a, d_fields, nfields, L.chunk_cap, s);
-  launch_decompress(a, n_total_capacity / kDChunkElems + nfields, s);
+  const uint64_t max_chunks = n_total_capacity / kDChunkElems + nfields;
+  launch_sizes(a, max_chunks, s);
+  launch_decompress(a, max_chunks, s);
   return launched();
 }
 

@@ -3,15 +3,14 @@
 // Persistent, warp-specialised CTAs; the roles hand chunks to one another through
 // mbarriers:
 //   header warp   takes a ticket, d1 reads the chunk's rate header, d2 derives the tile
-//                 sizes and scans them, publishes the chunk's aggregate flag at once and
-//                 leaves the chunk's record (headers, offsets, field parameters) in a ring
-//                 of records, running ahead of decoding;
-//   loader warp   d3 looks back for the chunk's byte offset (decoupled lookback) as soon
-//                 as the record is in, publishes the inclusive prefix, then takes the
-//                 chunk's payload bytes (its actual size, not the worst case) from a byte
-//                 ring, waiting for the oldest chunks' decoding to release space, and loads
-//                 the payload there with a 1-D TMA bulk copy. Compressed chunks being far
-//                 below the worst case, several are in flight per CTA;
+//                 sizes and scans them, d3 sums the sizes of the chunks before (computed
+//                 from the headers by the kernel before this one: no CTA waits for another)
+//                 and leaves the chunk's record (headers, offsets, field parameters) in a
+//                 ring of records, running ahead of decoding;
+//   loader warp   takes the chunk's payload bytes (its actual size, not the worst case)
+//                 from a byte ring, waiting for the oldest chunks' decoding to release
+//                 space, and loads the payload there with a 1-D TMA bulk copy. Compressed
+//                 chunks being far below the worst case, several are in flight per CTA;
 //   decode warps  (8) each decode a quad of 4 tiles at a time, lane L holding block L & 7
 //                 of tile L >> 3 (32 consecutive elements): d4 reads the block's sign map
 //                 and planes and undoes the bit shuffle with the register-pair delta swaps
@@ -43,16 +42,10 @@ static_assert(kDChunkTiles <= 32, "one lane per tile in the chunk scan");
 static_assert(kRingBytes % 16 == 0 && kRingBytes >= kMaxChunkRingBytes, "the ring holds the largest chunk");
 
 constexpr uint32_t kNoneChunk = 0xffffffffu;
-#ifndef FSZ_DEC_LOOKBACK_K
-#define FSZ_DEC_LOOKBACK_K 1
-#endif
-constexpr int kLookbackPerLane = FSZ_DEC_LOOKBACK_K;  // lookback window: 32 K flags
 // The schedule's work assignment (kernel arguments): a ticket hands a CTA ticket_chunks
 // consecutive chunks (at most kMaxTicketChunks). Their rate headers are read together,
-// and a chunk that follows its group's previous chunk in the same field takes its byte
-// offset from that chunk (no lookback), so the atomics and the lookbacks per chunk drop by
-// that factor. A CTA holds `records` chunks (2 x ticket_chunks .. kMaxRecs) between
-// ticket and decode.
+// and the group's byte offset is summed once. A CTA holds `records` chunks
+// (2 x ticket_chunks .. kMaxRecs) between ticket and decode.
 
 // A chunk's header and parameters, from the header warp to the loader and the decode
 // warps through shared memory (keeps dependent global loads off the decode path).
@@ -67,8 +60,7 @@ struct ChunkRec {
   uint64_t data_bytes;   // tile data bytes the preamble declares
   uint64_t data_base;    // 64 + 8T: start of the tile data
   uint64_t excl;         // byte offset of the chunk's payload in the tile data
-  uint32_t chunk;        // ticket, or kNoneChunk
-  uint32_t lc;           // chunk index inside the field
+  uint32_t chunk;        // global chunk index, or kNoneChunk
   uint32_t last;         // the field's last chunk
   uint32_t tot;          // payload bytes of the chunk
   uint32_t bad;          // reserved header bits seen
@@ -77,7 +69,6 @@ struct ChunkRec {
   uint32_t ntiles;
   uint32_t cnt;          // valid elements of the chunk
   uint32_t indep;        // the stream's blocks are independent (no carried state)
-  uint32_t chain;        // the previous record holds chunk - 1 of the same field
   float step;
 };
 
@@ -93,15 +84,6 @@ struct __align__(16) DecompressSmem {
 // two CTAs per SM (228 KiB of shared memory, 1 KiB of it reserved per CTA)
 static_assert(sizeof(DecompressSmem) <= 113 * 1024, "shared memory of one CTA");
 
-// Bytes of a tile from its 8 header bytes: sum of S_b (Eq. 3) + 4 for a centred tile.
-__device__ __forceinline__ uint32_t tile_bytes_from_header(uint64_t h) {
-  const uint64_t R = h & 0x1F1F1F1F1F1F1F1FULL;
-  const uint64_t W = R + (((R + 0x7F7F7F7F7F7F7F7FULL) & 0x8080808080808080ULL) >> 7);
-  const uint32_t lo = uint32_t(W), hi = uint32_t(W >> 32);
-  const uint32_t words = ((lo * 0x01010101u) >> 24) + ((hi * 0x01010101u) >> 24);
-  return 4u * words + ((h & 0x40u) ? 4u : 0u);
-}
-
 // Word offsets of the 8 blocks inside the tile's data (after mu), one per byte: the
 // exclusive byte-wise prefix sum of the blocks' word counts (rate + 1, or 0; <= 224).
 __device__ __forceinline__ uint64_t block_word_offsets(uint64_t h) {
@@ -112,6 +94,53 @@ __device__ __forceinline__ uint64_t block_word_offsets(uint64_t h) {
 
 __device__ __forceinline__ bool header_reserved_bits_set(uint64_t h) {
   return (h & 0x20u) || (h & 0xE0E0E0E0E0E0E000ULL);
+}
+
+// *p if `in`, else 0, read here: a plain load is moved down to its use by the compiler, past
+// the work that it is meant to run under. ld_now32 reads from L2.
+__device__ __forceinline__ uint64_t ld_now(const void* p, bool in) {
+  uint64_t v;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.u64 %0, 0;\n\t"
+      "@p ld.global.nc.u64 %0, [%1];\n\t}"
+      : "=l"(v)
+      : "l"(p), "r"(uint32_t(in)));
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_now32(const uint32_t* p, bool in) {
+  uint32_t v;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.u32 %0, 0;\n\t"
+      "@p ld.global.cg.u32 %0, [%1];\n\t}"
+      : "=r"(v)
+      : "l"(p), "r"(uint32_t(in)));
+  return v;
+}
+
+// The payload bytes of chunks lo .. hi - 1 are the sum over the warp of every lane's
+// range_lane_sum: the chunk sizes up to the first and from the last multiple of kSumBlock and
+// the block sums between, all loads independent. A CTA's tickets lie about one grid of
+// tickets apart, so a launch of 304 CTAs x 4 chunks reads 38 block sums and at most 62 sizes
+// per ticket; only a longer stretch needs the loop.
+constexpr int kRangeParts = 4;
+__device__ __forceinline__ void range_fetch(const uint32_t* sums, const uint32_t* block_sums,
+                                            uint64_t lo, uint64_t hi, uint32_t (&part)[kRangeParts],
+                                            uint64_t* rest) {
+  static_assert(kSumBlock == 32, "one lane per chunk of a block");
+  const int lane = threadIdx.x & 31;
+  const uint64_t b0 = (lo + 31) / 32, b1 = hi / 32;  // whole blocks b0 .. b1 - 1
+  const bool whole = b0 < b1;                        // (without one: at most 62 chunks)
+  const uint64_t k0 = lo + lane, k1 = (whole ? 32 * b1 : lo + 32) + lane;
+  part[0] = ld_now32(sums + k0, k0 < (whole ? 32 * b0 : hi));
+  part[1] = ld_now32(sums + k1, k1 < hi);
+  part[2] = ld_now32(block_sums + b0 + lane, b0 + lane < b1);
+  part[3] = ld_now32(block_sums + b0 + 32 + lane, b0 + 32 + lane < b1);
+  uint64_t v = 0;
+  for (uint64_t b = b0 + 64 + lane; b < b1; b += 32) v += ld_now32(block_sums + b, true);
+  *rest = v;
+}
+__device__ __forceinline__ uint64_t range_lane_sum(const uint32_t (&part)[kRangeParts], uint64_t rest) {
+  return rest + part[0] + part[1] + part[2] + part[3];  // (each below 2^22)
 }
 
 // Byte permute with the generic mode's sign replication (a selector nibble with bit 3 set
@@ -275,6 +304,42 @@ __device__ __forceinline__ bool decompress_quad(const uint64_t h, const uint64_t
   return __all_sync(FULL, good);
 }
 
+// The CTA's barrier 0, from whichever branch a warp is in.
+__device__ __forceinline__ void cta_sync() { asm volatile("barrier.sync 0;" ::: "memory"); }
+
+// What the header warp needs of a field.
+struct Field {
+  const uint8_t* sin;
+  float* dout;
+  uint64_t in_bytes, n, T, data_bytes;
+  uint64_t first;  // global index of the field's first chunk
+  uint32_t features_off;
+  float s;
+};
+
+__device__ __forceinline__ Field field_of_record(const FieldInfo* fi) {
+  return Field{fi->sin, fi->dout, fi->in_bytes, fi->n, fi->T, fi->data_bytes, fi->chunk_first,
+               fi->features_off, fi->s};
+}
+
+// The field of a one-field call, from the preamble as it stands: within the stream's buffer
+// and the output's capacity whatever it says.
+__device__ __forceinline__ Field field_of_stream(const KernelArgs& a) {
+  Field f = {};
+  f.sin = a.sin;
+  f.dout = a.dout;
+  f.in_bytes = a.in_bytes;
+  if (a.in_bytes < 64) return f;
+  const uint4* p = reinterpret_cast<const uint4*>(a.sin);
+  const uint4 w0 = p[0], w3 = p[3];
+  f.n = min(uint64_t(w0.z) | (uint64_t(w0.w) << 32), a.cap_elems);
+  f.T = min((f.n + kTile - 1) / kTile, (a.in_bytes - 64) / 8);
+  f.s = __uint_as_float(w3.x);
+  f.features_off = w3.y;
+  f.data_bytes = uint64_t(w3.z) | (uint64_t(w3.w) << 32);
+  return f;
+}
+
 // kAny: also decodes streams without the cross-block state. kPrezero: the output already
 // holds zeros; tiles whose 8 blocks all have rate 0 and no mean (all +0.0) are neither
 // decoded nor written (the adaptive pre-zero of Sec. 3.1 for high compression ratios).
@@ -295,120 +360,163 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
     }
     fence_mbar_init();
   }
-  grid_wait();
-  __syncthreads();
-
-  if (warp == kHeaderWarp) {
+  // (the header warp reads ahead before it waits)
+  if (warp != kHeaderWarp) {
+    grid_wait();
+    cta_sync();
+  } else {
     // ---------------------------------------------------------------- header warp
-    const uint64_t total = a.ctrl->total_chunks;
-    const uint32_t group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
-    const bool single = a.ctrl->nfields == 1;
-    for (uint32_t seq = 0;; seq += group) {
-      // the group's records must be free: their previous chunks decoded
-      bool ok = true;
-      for (uint32_t g = 0; g < group; ++g) {
-        const uint32_t sg = seq + g;
-        if (ok && sg >= recs) ok = mbar_wait(&S.done[sg % recs], ((sg / recs) - 1) & 1u, wait_ns);
+    // A ticket is a group of up to kMaxTicketChunks consecutive chunks; lane g keeps and writes
+    // what concerns chunk g as a whole, all lanes its tiles (lane = tile), the chunks side by
+    // side. This warp feeds all the others and shares their issue slots: with the chunks one
+    // after another and a ticket's atomic and loads in line it was the slowest stage. Whole
+    // calls before and after: 512^3 118.5 and 112.9 us, 16 M particles 29.5 and 24.6 us, batch
+    // of 32 fields 75.7 and 70.1 us.
+    const bool single = a.sin != nullptr;
+    Field f = {};        // lane g: chunk g's field (one field: the same in every lane)
+    uint64_t total = 0;  // chunks of the launch
+    uint64_t c0 = 0;     // the group's first chunk
+    uint32_t group = 1;
+    uint64_t h[kMaxTicketChunks];  // the lane's tile's header in each chunk, 0 beyond the field
+    uint32_t nt = 0;               // lane g: tiles of chunk g, 0 if there is none
+    uint32_t fidx = 0;             // lane g: chunk g's field
+    // the end of the previous group: the chunk after it, its offset in its field
+    uint64_t prev_end = 0, prev_excl = 0;
+    uint64_t from = 0;   // the group's offset is counted from here: the field's start or prev_end
+    uint32_t part[kRangeParts];
+    uint64_t part_rest = 0;
+    auto fetch_headers = [&]() {
+      const uint64_t c = c0 + lane;
+      const bool mine = uint32_t(lane) < group && c < total;
+      if (!single && mine) {
+        fidx = a.chunk_field[c];
+        f = field_of_record(a.fields + fidx);
       }
-      if (!ok) {
+      const uint64_t t0 = (c - f.first) * kDChunkTiles;
+      nt = mine ? uint32_t(min(uint64_t(kDChunkTiles), f.T - t0)) : 0u;
+      const uint64_t hp = reinterpret_cast<uint64_t>(f.sin) + 64 + 8 * t0;
+#pragma unroll
+      for (int g = 0; g < kMaxTicketChunks; ++g) {
+        const uint64_t p = __shfl_sync(FULL, hp, g);
+        h[g] = ld_now(reinterpret_cast<const unsigned long long*>(p) + lane,
+                      uint32_t(lane) < __shfl_sync(FULL, nt, g));
+      }
+    };
+    // d3: a CTA's chunks only go up, so the previous group ended in this one's field if it ended
+    // behind the field's first chunk
+    auto fetch_sizes = [&]() {
+      from = max(prev_end, __shfl_sync(FULL, f.first, 0));
+      range_fetch(a.sums, a.block_sums, from, c0 < total ? c0 : from, part, &part_rest);
+    };
+    if (single) {
+      // One field: its preamble and the headers of the CTA's first ticket (its own number) are
+      // read under the set-up kernel, which does not write them; what the preamble says counts
+      // only once that kernel's verdict (the control words' chunk count) is in.
+      f = field_of_stream(a);
+      total = (f.T + kDChunkTiles - 1) / kDChunkTiles;
+      group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
+      c0 = uint64_t(blockIdx.x) * group;
+      fetch_headers();
+    }
+    grid_wait();
+    cta_sync();
+    const uint64_t verdict = a.ctrl->total_chunks;
+    if (!single) {
+      total = verdict;
+      group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
+      c0 = uint64_t(blockIdx.x) * group;
+      fetch_headers();
+    }
+    fetch_sizes();
+    if (verdict == 0) nt = 0;
+    total = verdict;
+    for (uint32_t seq = 0;; seq += group) {
+      uint32_t next = 0;
+      if (lane == 0) next = gridDim.x + atomicAdd(&a.ctrl->ticket, 1u);
+      // the group's records must be free: their previous chunks decoded (the decode warps
+      // finish chunks in order, so the last record's tells)
+      const uint32_t sl = seq + group - 1;
+      if (sl >= recs && !mbar_wait(&S.done[sl % recs], ((sl / recs) - 1) & 1u, wait_ns)) {
         if (lane == 0) set_error(a.ctrl, nullptr, FSZ_ERR_TIMEOUT);
         return;
       }
-      // (tickets only go to running CTAs: a CTA that is not resident yet, e.g. behind
-      // another stream's kernel, holds no chunk that the others' lookbacks wait for)
-      uint32_t t = 0;
-      if (lane == 0) t = atomicAdd(&a.ctrl->ticket, 1u);
-      t = __shfl_sync(FULL, t, 0);
-      const uint64_t c0 = uint64_t(t) * group;
-      // field, position and rate header of each chunk of the group (loads issued together)
-      FieldInfo* fis[kMaxTicketChunks];
-      uint64_t hbs[kMaxTicketChunks];
+      // d2: tile sizes and their scans, the chunks side by side
+      uint32_t mine[kMaxTicketChunks], inc[kMaxTicketChunks], tot[kMaxTicketChunks];
+#pragma unroll
+      for (int g = 0; g < kMaxTicketChunks; ++g) inc[g] = mine[g] = tile_bytes_from_header(h[g]);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int g = 0; g < kMaxTicketChunks; ++g) inc[g] = scan_step_up<32>(inc[g], o);
+      // a tile may not use a feature the stream has switched off; streams without the
+      // cross-block state are decoded by the kAny instance only
+      const bool unsupported = !kAny && (f.features_off & kOffCross) && nt > 0;
+      if (unsupported) set_error(a.ctrl, a.fields + fidx, FSZ_ERR_INVALID_ARG);
+      const uint32_t forbid = ((f.features_off & kOffLz2) ? 0x80u : 0u) |
+                              ((f.features_off & kOffCenter) ? 0x40u : 0u);
+      uint32_t bad = unsupported ? 1u : 0u;
+      uint32_t my_tot = 0;
+      uint64_t excl = warp_sum_u64(range_lane_sum(part, part_rest)) +
+                      (prev_end > __shfl_sync(FULL, f.first, 0) ? prev_excl : 0);
+      uint64_t my_excl = 0;
+      const uint32_t starts = __ballot_sync(FULL, c0 + lane == f.first);  // bit g: a field's first chunk
 #pragma unroll
       for (int g = 0; g < kMaxTicketChunks; ++g) {
-        const uint64_t c = c0 + g;
-        fis[g] = nullptr;
-        hbs[g] = 0;
-        if (uint32_t(g) < group && c < total) {
-          FieldInfo* fi = single ? a.fields : a.fields + a.chunk_field[c];
-          fis[g] = fi;
-          const uint64_t tile0 = (c - fi->chunk_first) * kDChunkTiles;
-          if (tile0 + lane < fi->T)
-            hbs[g] = __ldg(reinterpret_cast<const unsigned long long*>(fi->sin + 64) + tile0 + lane);
+        tot[g] = __shfl_sync(FULL, inc[g], 31);
+        const uint32_t fb = __shfl_sync(FULL, forbid, g);
+        const bool b = __any_sync(FULL, header_reserved_bits_set(h[g]) || (uint32_t(h[g]) & fb) != 0);
+        if ((starts >> g) & 1u) excl = 0;
+        if (lane == g) {
+          my_tot = tot[g];
+          my_excl = excl;
+          if (b) bad = 1u;
         }
+        if (uint32_t(g) < group) excl += tot[g];
       }
-      bool end = false;
-      uint64_t prev_lc = 0;
+      // the records
+      uint32_t r = seq % recs, my_r = 0;
 #pragma unroll
       for (int g = 0; g < kMaxTicketChunks; ++g) {
-        if (uint32_t(g) >= group) break;
-        const uint32_t sg = seq + g;
-        const int r = int(sg % recs);
-        ChunkRec& q = S.rec[r];
-        const uint64_t c = c0 + g;
-        if (end) continue;
-        if (c >= total) {
-          if (lane == 0) {
-            q.chunk = kNoneChunk;
-            mbar_arrive(&S.fetched[r]);
-          }
-          end = true;
-          continue;
+        if (uint32_t(g) < group) {
+          ChunkRec& q = S.rec[r];
+          q.hdr[lane] = h[g];
+          q.boff[lane] = block_word_offsets(h[g]);
+          q.toff[lane] = inc[g] - mine[g];
+          if (lane == g) my_r = r;
+          if (++r == recs) r = 0;
         }
-        FieldInfo* fi = fis[g];
-        const uint64_t hb = hbs[g];
-        const uint64_t first = fi->chunk_first;
-        const uint64_t lc = c - first;
-        const uint64_t T = fi->T;
-        const uint64_t tile0 = lc * kDChunkTiles;
-        const int ntiles = int(min(uint64_t(kDChunkTiles), T - tile0));
-        if (lane < kDChunkTiles) {
-          q.hdr[lane] = hb;
-          q.boff[lane] = block_word_offsets(hb);
-        }
-        // a tile may not use a feature the stream has switched off
-        const uint32_t foff = fi->features_off;
-        const uint64_t forbid = ((foff & kOffLz2) ? 0x80u : 0u) | ((foff & kOffCenter) ? 0x40u : 0u);
-        // streams without the cross-block state are decoded by the kAny instance only
-        const bool unsupported = !kAny && (foff & kOffCross);
-        if (unsupported && lane == 0) set_error(a.ctrl, fi, FSZ_ERR_INVALID_ARG);
-        const bool bad_hdr = unsupported ||
-            __any_sync(FULL, lane < ntiles && (header_reserved_bits_set(hb) || (hb & forbid)));
-        const uint32_t mine = lane < ntiles ? tile_bytes_from_header(hb) : 0u;
-        uint32_t inc = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(FULL, inc, o);
-          if (lane >= o) inc += y;
-        }
-        if (lane < kDChunkTiles) q.toff[lane] = inc - mine;
-        const uint32_t tot = __shfl_sync(FULL, inc, 31);
-        // the chunk follows the group's previous one (unless that one is held back by the
-        // test hook, whose successors must meet its missing flag)
-        const bool chain = g > 0 && fis[g - 1] == fi && lc == prev_lc + 1 && c - 1 != a.skip_chunk;
-        prev_lc = lc;
-        if (lane == 0) {
-          if (c != a.skip_chunk) st_flag(a.flags + c * kFlagStride, (lc == 0 ? kFlagIncl : kFlagAgg) | tot);
-          q.chunk = uint32_t(c);
-          q.lc = uint32_t(lc);
-          q.last = (lc + 1 == fi->nchunks) ? 1u : 0u;
-          q.tot = tot;
-          q.bad = bad_hdr ? 1u : 0u;
-          q.fi = fi;
-          q.sin = fi->sin;
-          q.in_bytes = fi->in_bytes;
-          q.data_bytes = fi->data_bytes;
-          q.data_base = 64 + 8 * T;
-          q.dout = fi->dout + tile0 * kTile;
-          q.ntiles = uint32_t(ntiles);
-          q.cnt = uint32_t(min(fi->n - tile0 * kTile, uint64_t(kDChunkElems)));
-          q.step = fi->s;
-          q.indep = (foff & kOffCross) ? 1u : 0u;
-          q.chain = chain ? 1u : 0u;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&S.fetched[r]);
       }
-      if (end) return;
+      if (uint32_t(lane) < group) {
+        ChunkRec& q = S.rec[my_r];
+        const uint64_t t0 = (c0 + lane - f.first) * kDChunkTiles;
+        q.chunk = nt > 0 ? uint32_t(c0 + lane) : kNoneChunk;
+        q.last = t0 + kDChunkTiles >= f.T ? 1u : 0u;
+        q.tot = my_tot;
+        q.bad = bad;
+        q.fi = a.fields + fidx;
+        q.sin = f.sin;
+        q.in_bytes = f.in_bytes;
+        q.data_bytes = f.data_bytes;
+        q.data_base = 64 + 8 * f.T;
+        q.excl = my_excl;
+        q.dout = f.dout + t0 * kTile;
+        q.ntiles = nt;
+        q.cnt = uint32_t(min(f.n - t0 * kTile, uint64_t(kDChunkElems)));
+        q.step = f.s;
+        q.indep = (f.features_off & kOffCross) ? 1u : 0u;
+      }
+      __syncwarp();
+      // (test hook: the record of skip_chunk is never handed over, nor any after it)
+      const bool held = a.skip_chunk >= c0 && a.skip_chunk <= c0 + lane;
+      // ... and after the launch's last chunk one record says that there are no more
+      const uint32_t live = total > c0 ? uint32_t(min(total - c0, uint64_t(group))) : 0u;
+      if (uint32_t(lane) < group && !held && uint32_t(lane) <= live) mbar_arrive(&S.fetched[my_r]);
+      if (c0 + group > total || __any_sync(FULL, uint32_t(lane) < group && held)) return;
+      prev_end = c0 + group;
+      prev_excl = excl;
+      c0 = uint64_t(__shfl_sync(FULL, next, 0)) * group;
+      fetch_headers();
+      fetch_sizes();
     }
   }
 
@@ -419,7 +527,6 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
     // order, so the bytes in use are head - freed; pos is head's place in the ring.
     uint32_t head = 0, freed = 0, pos = 0;
     uint32_t oldest = 0;  // the oldest chunk whose bytes are not yet known to be released
-    uint64_t prev_excl = 0, prev_tot = 0;  // the previous record's chunk: offset and bytes
     for (uint32_t seq = 0;; ++seq) {
       const int r = int(seq % recs);
       if (!mbar_wait(&S.fetched[r], (seq / recs) & 1u, wait_ns)) {
@@ -427,31 +534,14 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
         return;
       }
       ChunkRec& q = S.rec[r];
-      const uint32_t c = q.chunk;
-      const bool none = c == kNoneChunk;
-      FieldInfo* fi = q.fi;
-      const uint32_t tot = q.tot;
-      const bool skip = !none && uint64_t(c) == a.skip_chunk;
-      uint64_t excl = 0;
-      if (!none && q.lc != 0) {
-        bool to = false;
-        if (q.chain)  // d3 from the group's previous chunk, resolved just before
-          excl = prev_excl + prev_tot;
-        else
-          excl = lookback<kLookbackPerLane>(a.flags, int64_t(c), int64_t(c) - int64_t(q.lc),
-                                            globaltimer_ns() + a.timeout_ns, &to);
-        if (lane == 0) {
-          if (to) set_error(a.ctrl, fi, FSZ_ERR_TIMEOUT);
-          if (!skip) st_flag(a.flags + uint64_t(c) * kFlagStride, kFlagIncl | (excl + tot));
-        }
-      }
-      prev_excl = excl;
-      prev_tot = tot;
-      if (none) {
+      if (q.chunk == kNoneChunk) {
         if (lane == 0) mbar_arrive(&S.full[r]);
         return;
       }
-      bool valid = q.bad == 0 && !skip;
+      FieldInfo* fi = q.fi;
+      const uint32_t tot = q.tot;
+      const uint64_t excl = q.excl;
+      bool valid = q.bad == 0;
       if (q.data_base + excl + tot > q.in_bytes) valid = false;
       if (q.last && excl + tot != q.data_bytes) valid = false;
       const uint64_t base = reinterpret_cast<uint64_t>(q.sin);
@@ -494,7 +584,7 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
       pos = phys + need;
       if (lane == 0) S.ring_end[r] = head;
       if (lane == 0) {
-        if (!valid && !skip) set_error(a.ctrl, fi, FSZ_ERR_CORRUPT);
+        if (!valid) set_error(a.ctrl, fi, FSZ_ERR_CORRUPT);
         q.pay = phys + uint32_t(src - a0);
         q.valid = valid ? 1u : 0u;
         if (bulk) {

@@ -113,6 +113,9 @@ struct alignas(64) Ctrl {
 };
 
 // Workspace layout: [Ctrl][FieldInfo x nfields][u32 chunk->field x cap][u64 flags x cap].
+// Decompression keeps its chunks' payload sizes (u32 x cap, and one sum per kSumBlock
+// chunks) where compression keeps its lookback flags.
+constexpr int kSumBlock = 32;
 struct WsLayout {
   uint64_t fields_off, map_off, flags_off, bytes;
   uint64_t chunk_cap;
@@ -132,13 +135,21 @@ struct KernelArgs {
   Ctrl* ctrl;
   FieldInfo* fields;
   const uint32_t* chunk_field;
-  uint64_t* flags;
-  uint64_t skip_chunk;  // test hook: this chunk publishes no flag
+  uint64_t* flags;       // compression: lookback flags
+  uint32_t* sums;        // decompression: payload bytes of each chunk,
+  uint32_t* block_sums;  // ... and of each kSumBlock consecutive ones
+  uint64_t skip_chunk;  // test hook: this chunk publishes no flag (decompression: no record)
   uint64_t timeout_ns;  // bound on every spin-wait
   // multipass compression only: the four variants' tile costs, variant-major (given_T
   // per variant), from which the encoding pass selects
   const uint32_t* given_costs = nullptr;
   uint64_t given_T = 0;
+  // decompression of one field: the stream and the output (null for a batch), which the
+  // kernel reads and places without going through the field record
+  const uint8_t* sin = nullptr;
+  uint64_t in_bytes = 0;
+  float* dout = nullptr;
+  uint64_t cap_elems = 0;
   // work assignment (from the schedule, set by the launch functions)
   uint32_t ticket_chunks = 1;  // consecutive chunks per ticket
   uint32_t ticket_lead = 1;    // compression: tickets taken ahead of the compute warps
@@ -486,6 +497,17 @@ __device__ __forceinline__ uint64_t lookback(const uint64_t* flags, int64_t gchu
   return excl;
 }
 
+// ------------------------------------------------------------------ rate headers
+
+// Bytes of a tile from its 8 header bytes: sum of S_b (Eq. 3) + 4 for a centred tile.
+__device__ __forceinline__ uint32_t tile_bytes_from_header(uint64_t h) {
+  const uint64_t R = h & 0x1F1F1F1F1F1F1F1FULL;
+  const uint64_t W = R + (((R + 0x7F7F7F7F7F7F7F7FULL) & 0x8080808080808080ULL) >> 7);
+  const uint32_t lo = uint32_t(W), hi = uint32_t(W >> 32);
+  const uint32_t words = ((lo * 0x01010101u) >> 24) + ((hi * 0x01010101u) >> 24);
+  return 4u * words + ((h & 0x40u) ? 4u : 0u);
+}
+
 // ------------------------------------------------------------------ float keys
 
 __device__ __forceinline__ uint32_t float_key(float x) {
@@ -624,11 +646,12 @@ void launch_cost_pass(const KernelArgs& a, int variant, uint32_t* costs, cudaStr
 enum DecompressKind { kDecompressFull = 0, kDecompressAny = 1, kDecompressPrezeroed = 2 };
 void launch_decompress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st,
                        DecompressKind kind = kDecompressFull);
-// Single-field set-up (clears the control words, the field record and chunk_cap lookback
-// flags of the workspace, then fills in the field): no memset of the workspace needed.
+// Single-field set-up: fills in the control words and the field record; for compression it
+// clears the lookback flags, for decompression it sizes the chunks' payloads (no memset of
+// the workspace needed). launch_sizes: the sizing of a planned batch.
 void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t chunk_cap, cudaStream_t st);
-void launch_setup_decompress(const KernelArgs& a, const uint8_t* in, uint64_t in_bytes, float* out,
-                             uint64_t cap_elems, uint64_t chunk_cap, cudaStream_t st);
+void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st);
+void launch_sizes(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st);
 void launch_plan_compress(const KernelArgs& a, const fsz_cfield* d_fields, uint32_t nfields,
                           uint64_t chunk_cap, cudaStream_t st);
 void launch_plan_decompress(const KernelArgs& a, const fsz_dfield* d_fields, uint32_t nfields,

@@ -219,6 +219,14 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
   }
 }
 
+// n *= dk; false if the product exceeds kMaxElems (n itself does not). Without a 64-bit
+// division, which the single thread that plans a field would wait for.
+__device__ __forceinline__ bool times_dim(uint64_t* n, uint64_t dk) {
+  if (__umul64hi(*n, dk) != 0) return false;
+  *n *= dk;
+  return *n <= kMaxElems;
+}
+
 // Validates one compression descriptor and fills the field's shape (host-visible errors
 // of the one-field entry point are checked again here for batches).
 __device__ uint32_t plan_cfield(FieldInfo* fi, const fsz_cfield& d) {
@@ -237,8 +245,7 @@ __device__ uint32_t plan_cfield(FieldInfo* fi, const fsz_cfield& d) {
   uint64_t n = 1;
   for (uint32_t k = 0; k < d.dims.ndim; ++k) {
     const uint64_t dk = d.dims.dims[k];
-    if (dk != 0 && n > kMaxElems / dk) return FSZ_ERR_INVALID_ARG;
-    n *= dk;
+    if (!times_dim(&n, dk)) return FSZ_ERR_INVALID_ARG;
     fi->dims[k] = dk;
   }
   if (n > kMaxElems) return FSZ_ERR_INVALID_ARG;
@@ -283,8 +290,7 @@ __device__ uint32_t plan_dfield(FieldInfo* fi, const uint8_t* in, uint64_t in_by
       if (dk != 0) return FSZ_ERR_CORRUPT;
       continue;
     }
-    if (dk != 0 && prod > kMaxElems / dk) return FSZ_ERR_CORRUPT;
-    prod *= dk;
+    if (!times_dim(&prod, dk)) return FSZ_ERR_CORRUPT;
     fi->dims[k] = dk;
   }
   if (prod != n || n > kMaxElems) return FSZ_ERR_CORRUPT;
@@ -319,7 +325,7 @@ __device__ void finish_empty_field(Ctrl* ctrl, FieldInfo* fi) {
 
 // One-field set-up for compression: the descriptor is validated on the host, so this
 // copies it into the workspace.
-// Set-up of a single-field call: thread 0 of CTA 0 clears the control words and the field
+// Set-up of a single-field compression: thread 0 of CTA 0 clears the control words and the field
 // record and fills them in; every other thread clears the lookback flags (nflags words),
 // so that the call needs no separate memset.
 constexpr int kSetupThreads = 256;
@@ -358,20 +364,129 @@ __global__ void __launch_bounds__(kSetupThreads) fsz_setup_compress_kernel(Kerne
   if (desc.n == 0) finish_empty_field(a.ctrl, fi);
 }
 
-__global__ void __launch_bounds__(kSetupThreads) fsz_setup_decompress_kernel(
-    KernelArgs a, const uint8_t* in, uint64_t in_bytes, float* out, uint64_t cap_elems,
-    uint64_t chunk_cap, uint64_t nflags) {
-  if (!setup_clear(a, nflags)) return;
-  FieldInfo* fi = a.fields;
-  uint32_t st = plan_dfield(fi, in, in_bytes, out, cap_elems);
-  if (st == FSZ_OK && fi->nchunks > chunk_cap) st = FSZ_ERR_WORKSPACE;
-  if (st != FSZ_OK) {
-    set_error(a.ctrl, fi, st);
-    fi->nchunks = 0;
+// Payload sizes of the chunks, from the rate headers alone (8 of them per 32 KiB of output):
+// one warp per chunk, one CTA per kSumBlock chunks at a time. A chunk's byte offset is then
+// a short sum over these (range_fetch in the decompression kernel), where a decoupled
+// lookback during decompression made the first chunk of each CTA wait 5 to 11 us for the
+// others. Bound by latency (two loads and two barriers); with the set-up 4.3 us at 512^3
+// (4 MB of headers), 3.3 us at 2^20 values, against 3.1 and 2.7 us for the set-up alone.
+// 16 warps with two chunks each: 32 warps with one took 7.8 us at 512^3.
+constexpr int kSizeWarps = 16;
+constexpr int kSizeThreads = 32 * kSizeWarps;
+constexpr int kChunksPerWarp = kSumBlock / kSizeWarps;  // of a block: warp, warp + kSizeWarps
+
+// Records the sizes of one block of chunks; bytes[k]: this lane's tile of chunk
+// kSumBlock * block + kSizeWarps * k + warp (0 beyond the last tile).
+__device__ __forceinline__ void write_chunk_sizes(const KernelArgs& a, uint64_t block, uint64_t total,
+                                                  const uint32_t (&bytes)[kChunksPerWarp],
+                                                  uint32_t* s_sum) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < kChunksPerWarp; ++k) {
+    const uint64_t c = block * kSumBlock + kSizeWarps * k + warp;
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, bytes[k]);
+    if (lane == 0) {
+      s_sum[kSizeWarps * k + warp] = sum;
+      if (c < total) a.sums[c] = sum;
+    }
   }
-  fi->chunk_first = 0;
-  a.ctrl->nfields = 1;
-  a.ctrl->total_chunks = fi->nchunks;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, s_sum[lane]);
+    if (lane == 0) a.block_sums[block] = sum;
+  }
+  __syncthreads();
+}
+
+// One field: sized beside the parsing of its preamble (by one thread of CTA 0) rather than
+// after it. The element count is read from the preamble as it stands, bounded by the
+// output's capacity, and the headers within the stream's buffer; the sizes of a stream that
+// the parsing refuses are not used.
+__global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(
+    KernelArgs a, uint64_t chunk_cap) {
+  const uint8_t* const in = a.sin;
+  const uint64_t in_bytes = a.in_bytes, cap_elems = a.cap_elems;
+  __shared__ uint32_t s_sum[kSumBlock];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  grid_wait();
+  grid_release();
+  const unsigned long long* const hdr = reinterpret_cast<const unsigned long long*>(in + 64);
+  const uint64_t n = in_bytes >= 64 ? *reinterpret_cast<const uint64_t*>(in + 8) : 0;
+  const uint64_t readable = in_bytes >= 64 ? (in_bytes - 64) / 8 : 0;  // whole headers in the buffer
+  auto tile = [&](uint64_t b, int k) {
+    return (b * kSumBlock + kSizeWarps * k + warp) * kDChunkTiles + lane;
+  };
+  uint64_t h[kChunksPerWarp];
+#pragma unroll
+  for (int k = 0; k < kChunksPerWarp; ++k) {  // (issued with n's load)
+    const uint64_t t = tile(blockIdx.x, k);
+    h[k] = t < readable ? __ldg(hdr + t) : 0;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    FieldInfo f = {};
+    uint32_t st = plan_dfield(&f, in, in_bytes, a.dout, cap_elems);
+    if (st == FSZ_OK && f.nchunks > chunk_cap) st = FSZ_ERR_WORKSPACE;
+    if (st != FSZ_OK) f.nchunks = 0;
+    f.status = st;
+    Ctrl c = {};
+    c.status = st;
+    c.nfields = 1;
+    c.total_chunks = f.nchunks;
+    *a.fields = f;
+    *a.ctrl = c;
+  }
+  const uint64_t T = min((min(n, cap_elems) + kTile - 1) / kTile, readable);
+  const uint64_t total = (T + kDChunkTiles - 1) / kDChunkTiles;  // <= chunk_cap
+  for (uint64_t b = blockIdx.x; b * kSumBlock < total; b += gridDim.x) {
+    uint32_t bytes[kChunksPerWarp];
+#pragma unroll
+    for (int k = 0; k < kChunksPerWarp; ++k) {
+      const uint64_t t = tile(b, k);
+      if (b != blockIdx.x) h[k] = t < T ? __ldg(hdr + t) : 0;
+      bytes[k] = t < T ? tile_bytes_from_header(h[k]) : 0u;
+    }
+    write_chunk_sizes(a, b, total, bytes, s_sum);
+  }
+}
+
+// A planned batch.
+__global__ void __launch_bounds__(kSizeThreads) fsz_sizes_kernel(KernelArgs a) {
+  __shared__ uint32_t s_sum[kSumBlock];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  grid_wait();
+  grid_release();
+  const uint64_t total = a.ctrl->total_chunks;
+  for (uint64_t b = blockIdx.x; b * kSumBlock < total; b += gridDim.x) {
+    uint32_t bytes[kChunksPerWarp];
+#pragma unroll
+    for (int k = 0; k < kChunksPerWarp; ++k) {
+      const uint64_t c = b * kSumBlock + kSizeWarps * k + warp;
+      bytes[k] = 0;
+      if (c < total) {
+        const FieldInfo* fi = a.fields + a.chunk_field[c];
+        const uint64_t t = (c - fi->chunk_first) * kDChunkTiles + lane;
+        if (t < fi->T)
+          bytes[k] = tile_bytes_from_header(
+              __ldg(reinterpret_cast<const unsigned long long*>(fi->sin + 64) + t));
+      }
+    }
+    write_chunk_sizes(a, b, total, bytes, s_sum);
+  }
+}
+
+// CTAs of a sizing launch: one per kSumBlock chunks, at most four per SM.
+int sizes_grid(uint64_t max_chunks) {
+  static DeviceCfgCache cache;
+  const LaunchCfg c = cache.get([] {
+    LaunchCfg cfg = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&cfg.sms, cudaDevAttrMultiProcessorCount, dev);
+    cfg.grid = 4 * cfg.sms;
+    return cfg;
+  });
+  const uint64_t g = (max_chunks + kSumBlock - 1) / kSumBlock;
+  return g < uint64_t(c.grid) ? int(g > 0 ? g : 1) : c.grid;
 }
 
 // CTAs of a set-up launch: one plus one per 2048 flag words, at most 152.
@@ -499,11 +614,14 @@ void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t ch
   launch_dependent(fsz_setup_compress_kernel, setup_grid(nflags), kSetupThreads, 0, st, a, fi, nflags);
 }
 
-void launch_setup_decompress(const KernelArgs& a, const uint8_t* in, uint64_t in_bytes, float* out,
-                             uint64_t cap_elems, uint64_t chunk_cap, cudaStream_t st) {
-  const uint64_t nflags = kFlagStride * chunk_cap;
-  launch_dependent(fsz_setup_decompress_kernel, setup_grid(nflags), kSetupThreads, 0, st, a, in,
-                   in_bytes, out, cap_elems, chunk_cap, nflags);
+void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st) {
+  launch_dependent(fsz_setup_decompress_kernel,
+                   sizes_grid((a.cap_elems + kDChunkElems - 1) / kDChunkElems), kSizeThreads, 0, st, a,
+                   chunk_cap);
+}
+
+void launch_sizes(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st) {
+  launch_dependent(fsz_sizes_kernel, sizes_grid(max_chunks), kSizeThreads, 0, st, a);
 }
 
 void launch_plan_compress(const KernelArgs& a, const fsz_cfield* d_fields, uint32_t nfields,
