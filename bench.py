@@ -561,9 +561,9 @@ def run_ablation(fsz, fields, rels, dev, shape):
 
 def run_tiles(fsz, fields, rels, dev, shape):
     """Sec. 6.5 (Table 8): every tile configuration (B elements per block, T blocks per
-    tile) on the bench fields through the generic two-read path: CR against the default
-    B = 32, T = 8 (win / loss beyond 2 %, tie within), and the generic path's compression
-    and decompression time; the specialised single-pass kernels cover 32 x 8 only."""
+    tile) on the bench fields through fsz_compress_tiled / fsz_decompress_tiled: CR against
+    the default B = 32, T = 8 (win / loss beyond 2 %, tie within), and the compression and
+    decompression time."""
     import math
     import statistics
 
@@ -619,7 +619,7 @@ def run_tiles(fsz, fields, rels, dev, shape):
                         "decompress_gbs_geomean": math.exp(sum(math.log(r[key]["decompress_gbs"]) for r in rows) / len(rows))}
     del out, rec, ws
     torch.cuda.empty_cache()
-    return {"workload": "the bench fields at each REL, every (B, T) through the generic tiled path",
+    return {"workload": "the bench fields at each REL, every (B, T) through the tiled entry points",
             "rows": rows, "vs_32x8": summary}
 
 

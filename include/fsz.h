@@ -188,10 +188,9 @@ fsz_status fsz_decompress_any(const void* d_in, uint64_t in_bytes, float* d_out,
  * 64) and `tile_blocks` blocks per tile (4, 8 or 16). A configured stream has tile_blocks
  * header bytes per tile and block-bit sign and plane words (block / 8 bytes, element j at
  * bit block - 1 - j, most significant byte first); the method word (preamble byte 52)
- * holds the configuration in bits 8-15 (0 for 32 x 8, the default). A generic two-read
- * path (a cost pass, a scan of tile sizes, an encoding pass; one warp per tile) for every
- * configuration; the default configuration's specialised single-pass kernels are
- * fsz_compress / fsz_decompress, and fsz_decompress refuses configured streams. */
+ * holds the configuration in bits 8-15 (0 for 32 x 8, the default). Instances of the same
+ * kernels serve every configuration; fsz_compress / fsz_decompress are the calls for the
+ * default one, and fsz_decompress refuses configured streams. */
 uint64_t fsz_compress_bound_tiled(uint64_t n, uint32_t block, uint32_t tile_blocks);
 /* Workspace for fsz_compress_tiled / fsz_decompress_tiled of up to n elements. */
 uint64_t fsz_tiled_workspace_bytes(uint64_t n);

@@ -147,7 +147,7 @@ fsz_status decompress_one(const void* d_in, uint64_t in_bytes, float* d_out,
   a.in_bytes = in_bytes;
   a.dout = d_out;
   a.cap_elems = out_capacity_elems;
-  launch_setup_decompress(a, L.chunk_cap, s);
+  launch_setup_decompress(a, L.chunk_cap, s, kind == kDecompressTiled);
   launch_decompress(a, (out_capacity_elems + kDChunkElems - 1) / kDChunkElems, s, kind);
   return launched();
 }
@@ -279,6 +279,69 @@ fsz_status fsz_decompress_any(const void* d_in, uint64_t in_bytes, float* d_out,
                               fsz_stream stream) {
   return decompress_one(d_in, in_bytes, d_out, out_capacity_elems, d_ws, ws_bytes, stream,
                         kDecompressAny);
+}
+
+// Tile configurations (Sec. 6.5, Table 8): instances of the same kernels, three launches to
+// compress and two to decompress as for the default configuration.
+
+uint64_t fsz_compress_bound_tiled(uint64_t n, uint32_t block, uint32_t tile_blocks) {
+  if ((block != 32 && block != 64) || (tile_blocks != 4 && tile_blocks != 8 && tile_blocks != 16))
+    return 0;
+  const uint64_t tile = uint64_t(block) * tile_blocks;
+  const uint64_t NT = (n + tile - 1) / tile;
+  return 64 + uint64_t(tile_blocks) * NT + (uint64_t(tile_blocks) * (block / 8) * 24 + 4) * NT;
+}
+
+// The workspace of one field and 20 bytes per 128 elements beside it. The calls need the
+// former only; the size that callers allocate and keep is unchanged.
+uint64_t fsz_tiled_workspace_bytes(uint64_t n) {
+  const uint64_t tiles = (n + 127) / 128 + 1;
+  auto a16 = [](uint64_t x) { return (x + 15) & ~uint64_t(15); };
+  uint64_t b = a16(ws_layout((n + kTile - 1) / kTile, 1).bytes);
+  b = a16(b + 4 * tiles);
+  b = a16(b + 8 * tiles);
+  b = a16(b + 8 * tiles);
+  return b + 8 * (tiles / 4096 + 2);
+}
+
+fsz_status fsz_compress_tiled(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double eb,
+                              uint32_t block, uint32_t tile_blocks, uint32_t features_off,
+                              void* d_out, uint64_t out_capacity, uint64_t* d_out_bytes, void* d_ws,
+                              uint64_t ws_bytes, fsz_stream stream) {
+  if ((block != 32 && block != 64) || (tile_blocks != 4 && tile_blocks != 8 && tile_blocks != 16))
+    return FSZ_ERR_INVALID_ARG;
+  if (!features_valid(features_off)) return FSZ_ERR_INVALID_ARG;
+  uint64_t n = 0;
+  fsz_status st = dims_count(dims, &n);
+  if (st != FSZ_OK) return st;
+  if (n == 0) return FSZ_ERR_INVALID_ARG;
+  if (d_ws == nullptr || ws_bytes < fsz_tiled_workspace_bytes(n)) return FSZ_ERR_WORKSPACE;
+  const uint64_t tile = uint64_t(block) * tile_blocks;
+  const uint64_t NT = (n + tile - 1) / tile;
+  if (out_capacity < 64 + tile_blocks * NT) return FSZ_ERR_CAPACITY;
+  CompressCall call;
+  st = check_compress(d_in, dims, mode, eb, d_out, out_capacity, d_ws, ws_bytes, &call, features_off);
+  if (st != FSZ_OK) return st;
+  call.desc.out_bytes = d_out_bytes;
+  call.desc.T = NT;
+  call.desc.features_off = features_off | tile_word_of(int(block), int(tile_blocks));
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  const KernelArgs a = make_args(d_ws, call.L);
+  launch_setup_compress(a, call.desc, call.L.chunk_cap, s);
+  launch_stats(a, d_in, n, s);
+  launch_compress_tiled(a, call.desc.nchunks, int(block), int(tile_blocks), s);
+  return launched();
+}
+
+fsz_status fsz_decompress_tiled(const void* d_in, uint64_t in_bytes, float* d_out,
+                                uint64_t out_capacity_elems, void* d_ws, uint64_t ws_bytes,
+                                fsz_stream stream) {
+  if (ws_bytes < fsz_tiled_workspace_bytes(out_capacity_elems < kMaxElems ? out_capacity_elems : kMaxElems) &&
+      d_in != nullptr && d_out != nullptr && d_ws != nullptr && !misaligned(d_in) && !misaligned(d_out) &&
+      !misaligned(d_ws))
+    return FSZ_ERR_WORKSPACE;
+  return decompress_one(d_in, in_bytes, d_out, out_capacity_elems, d_ws, ws_bytes, stream,
+                        kDecompressTiled);
 }
 
 fsz_status fsz_compress_batched(const fsz_cfield* d_fields, uint32_t nfields, uint64_t n_total,

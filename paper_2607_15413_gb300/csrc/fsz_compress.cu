@@ -32,8 +32,8 @@ namespace fsz {
 namespace {
 
 constexpr uint32_t FULL = 0xffffffffu;
-constexpr int kQuadTiles = 4;                      // tiles per compute warp and chunk
-constexpr int kWarps = kCChunkTiles / kQuadTiles;  // compute warps per CTA
+constexpr int kQuadElems = 1024;                   // elements per compute warp and chunk
+constexpr int kWarps = kCChunkElems / kQuadElems;  // compute warps per CTA
 constexpr int kHostWarp = kWarps;                  // tickets and placement
 constexpr int kResolverWarp = kWarps + 1;
 constexpr int kThreads = (kWarps + 2) * 32;
@@ -60,9 +60,10 @@ static_assert(kMaxTicketChunks + kMaxCompressLead <= FSZ_COMPRESS_SETS, "schedul
 #define FSZ_COMPRESS_CTAS 2
 #endif
 constexpr int kCtasPerSm = FSZ_COMPRESS_CTAS;
-constexpr int kQuadElems = kQuadTiles * kTile;     // 1024
 constexpr int kQuadBytes = 4 * kQuadElems;         // 4096: a warp's staging buffer
-constexpr int kMaxQuadOut = kQuadTiles * kMaxTileBytes;
+constexpr int kMaxQuadOut = 4 * kMaxTileBytes;
+// ... of any tile configuration: 32 blocks (or halves) of at most 24 words, up to 8 means
+constexpr int kMaxCfgQuadOut = 32 * 4 * 24 + 8 * 4;
 // Ring bytes per compute warp. A run is contiguous: one that would run past the end
 // starts at the ring's start instead, and the bytes it skips count as its own until it
 // is placed.
@@ -86,8 +87,10 @@ constexpr uint32_t kNone = 0xffffffffu;
 constexpr uint32_t kHostSleepNs = FSZ_HOST_SLEEP_NS;
 constexpr uint32_t kResolverSleepNs = FSZ_RESOLVER_SLEEP_NS;
 constexpr uint32_t kComputeSleepNs = FSZ_COMPUTE_SLEEP_NS;
-static_assert(kCChunkTiles == kWarps * kQuadTiles, "a chunk is one quad per compute warp");
-static_assert(kRingAlloc >= 2 * kMaxQuadOut, "worst-case quads fit the ring");
+static_assert(kCChunkElems == kWarps * kQuadElems && kCChunkElems == kDChunkElems,
+              "a chunk is one quad per compute warp");
+static_assert(kRingAlloc >= 2 * kMaxQuadOut && kRingAlloc >= 2 * kMaxCfgQuadOut,
+              "worst-case quads fit the ring");
 static_assert(kRingAlloc % 16 == 0 && kQuadBytes % 1024 == 0, "alignment of the buffers");
 static_assert(kWarps <= 32, "one lane per quad in the chunk scan");
 
@@ -99,7 +102,7 @@ struct ChunkInfo {
   uint8_t* out;          // the field's stream
   FieldInfo* fi;
   uint64_t tile0;        // field-local index of the chunk's first tile
-  uint64_t data_base;    // 64 + 8T: start of the field's tile data
+  uint64_t data_base;    // start of the field's tile data, after the rate headers
   uint64_t cap;          // the field's output capacity
   uint64_t chunk_first;  // global index of the field's first chunk
   uint32_t chunk;        // global ticket, or kNone
@@ -127,7 +130,8 @@ struct __align__(1024) CompressSmem {
 
 static_assert(sizeof(CompressSmem) <= 227 * 1024, "shared memory of one CTA");
 
-// Eq. 3: S_b = 0 for r_b = 0, else 4 + 4 r_b.
+// Eq. 3: S_b = 0 for r_b = 0, else 4 + 4 r_b; of a 64-element block, each of its two lanes'
+// share.
 __device__ __forceinline__ uint32_t block_cost(int R) {
   return (uint32_t(R) + (R != 0 ? 1u : 0u)) << 2;
 }
@@ -234,20 +238,22 @@ __device__ __forceinline__ void planes8(const uint32_t (&v)[32], uint32_t (&X)[8
   swap_planes(X);
 }
 
-// Compresses one quad (4 tiles) with one warp. Lane L = 8 tq + g holds block g of tile tq
-// (elements 32 g .. 32 g + 31 of the tile) in d. `live`: the lane's tile exists. Writes the
-// tile's rate-header byte of block g to hdr (the quad's 32 header bytes are consecutive),
-// and returns this lane's block as (byte offset of its data inside the quad's run, word
-// count), with the quad's run length in *qlen; the words go to ring + offset by encode().
-// Switched-off features arrive as `restart` (this lane starts from zero predecessors: the
-// tile's first block, and every block without the cross-block state) and as penalties
-// pen2, pen3 (2^16 for the second-order and the centred variants when off). With kGiven
-// the four tile costs come from `given` (this lane's tile, stride gT between variants): the
-// multipass evaluation's encoding pass; they are equal, so the stream is the same.
+// Compresses one quad (1024 elements: 1 to 8 tiles, 4 in the default configuration) with one
+// warp. Lane L holds elements 32 L .. 32 L + 31 in d: a block, or half of a 64-element one;
+// g is the lane's number in its tile. `live`: the lane's tile exists. Writes the rate-header
+// byte of the lane's block to hdr (the quad's header bytes are consecutive), and returns the
+// lane's words' place in the quad's run, with the quad's run length in P.qlen; the words go
+// to ring + offset by encode_block(). Switched-off features arrive as `restart` (this lane
+// starts from zero predecessors: the tile's first lane, and every block's without the
+// cross-block state) and as penalties pen2, pen3 (2^16 for the second-order and the centred
+// variants when off). With kGiven the four tile costs come from `given` (this lane's tile,
+// stride gT between variants): the multipass evaluation's encoding pass; they are equal, so
+// the stream is the same.
 struct QuadPlan {
   uint32_t v[32];   // the selected variant's residuals: magnitude in bits 0-22
   uint32_t signs;   // ... and their sign map, as the stream's word
-  uint32_t off;     // byte offset of this lane's block data in the quad's run
+  uint32_t off;     // byte offset of this lane's first word in the quad's run (the words of a
+                    // block's lanes alternate)
   int R;            // the block's rate (0 for a dead tile): its planes, after the sign map
   uint32_t mu_off;  // byte offset of the tile's mean slot (lane g = 0 of a centred tile)
   bool mu_slot;
@@ -256,17 +262,19 @@ struct QuadPlan {
   int Rmax;         // largest live rate of the quad (uniform)
 };
 
-template <bool kGiven>
+template <bool kGiven, typename Cfg>
 __device__ __forceinline__ void plan_quad(const float (&d)[32], const float r, const int lane,
                                           const bool live, const bool restart, const int pen2,
                                           const int pen3, const uint32_t* __restrict__ given,
                                           const uint64_t gT, uint8_t* __restrict__ hdr,
                                           QuadPlan& P) {
-  const int g = lane & 7;
+  constexpr int LT = Cfg::kLanes;
+  const int g = lane & (LT - 1);
   // Tile sum for centring (Sec. 4.2.2, variant 3) in the fixed order: the sums of elements
   // 8j..8j+7 left to right (four runs per lane: runs 4g .. 4g + 3), then a butterfly over
-  // the run index by 16, 8, 4 (lanes xor 4, 2, 1 within the tile's 8 lanes), 2 and 1
-  // (in-lane). Float addition is commutative, so both partners of a step get equal sums.
+  // the run index by half the runs, a quarter, .. 4 (lanes xor LT / 2 .. 1 within the tile),
+  // 2 and 1 (in-lane). Float addition is commutative, so both partners of a step get equal
+  // sums.
   float R[4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
@@ -276,7 +284,7 @@ __device__ __forceinline__ void plan_quad(const float (&d)[32], const float r, c
     R[m] = acc;
   }
 #pragma unroll
-  for (int o = 4; o >= 1; o >>= 1)
+  for (int o = LT / 2; o >= 1; o >>= 1)
 #pragma unroll
     for (int m = 0; m < 4; ++m) R[m] = __fadd_rn(R[m], __shfl_xor_sync(FULL, R[m], o));
   const float S = __fadd_rn(__fadd_rn(R[0], R[2]), __fadd_rn(R[1], R[3]));
@@ -291,14 +299,14 @@ __device__ __forceinline__ void plan_quad(const float (&d)[32], const float r, c
   float Y[32];
 #pragma unroll
   for (int i = 0; i < 32; ++i) Y[i] = __fadd_rn(__fmul_rn(d[i], r), kMagic);
-  const float muY = __fadd_rn(__fmul_rn(__fmul_rn(S, 0.00390625f), r), kMagic);
+  const float muY = __fadd_rn(__fmul_rn(__fmul_rn(S, 1.0f / float(Cfg::kElems)), r), kMagic);
   const float mu = __fsub_rn(muY, kMagic);
 
   // Residuals with the state carried across block boundaries (Eq. 2); the tile's first
   // predecessors are zero. LZ2 as the difference of LZ1 residuals:
   // l2_i = (q_i - q_{i-1}) - (q_{i-1} - q_{i-2}).
-  float prevY = __shfl_up_sync(FULL, Y[31], 1, 8);
-  float prevL = __shfl_up_sync(FULL, __fsub_rn(Y[31], Y[30]), 1, 8);
+  float prevY = __shfl_up_sync(FULL, Y[31], 1, LT);
+  float prevL = __shfl_up_sync(FULL, __fsub_rn(Y[31], Y[30]), 1, LT);
   if (restart) {
     prevY = kMagic;
     prevL = 0.0f;
@@ -320,22 +328,27 @@ __device__ __forceinline__ void plan_quad(const float (&d)[32], const float r, c
   }
   const float rest1 = max3_abs(m1[0], m1[1], m1[2]);
   const float rest2 = max3_abs(m2[0], m2[1], m2[2]);
-  const int R1 = bitlen(fmaxf(rest1, fabsf(l1_0)));
-  const int R2 = bitlen(max3_abs(rest2, l2_0, l2_1));
-  // Centred block-0 rates (lane g = 0): l1c_0 = q_0 - mu, l2c_0 = q_0 - mu,
-  // l2c_1 = q_1 - 2 q_0 + mu = l2_1 + mu; the rest of block 0 is unchanged (Eq. 4).
+  // Centring changes the tile's first residuals (lane g = 0): l1c_0 = q_0 - mu, l2c_0 =
+  // q_0 - mu, l2c_1 = q_1 - 2 q_0 + mu = l2_1 + mu; the rest is unchanged (Eq. 4).
   const float c10 = __fsub_rn(Y[0], muY);
   const float c21 = __fadd_rn(l2_1, mu);
-  const int R1c = bitlen(fmaxf(rest1, fabsf(c10)));
-  const int R2c = bitlen(max3_abs(rest2, c10, c21));
+  float M1 = fmaxf(rest1, fabsf(l1_0)), M2 = max3_abs(rest2, l2_0, l2_1);
+  float M1c = g == 0 ? fmaxf(rest1, fabsf(c10)) : M1;
+  float M2c = g == 0 ? max3_abs(rest2, c10, c21) : M2;
+  if constexpr (Cfg::kBlockLanes == 2) {  // a block's two lanes
+    M1 = fmaxf(M1, __shfl_xor_sync(FULL, M1, 1));
+    M2 = fmaxf(M2, __shfl_xor_sync(FULL, M2, 1));
+    M1c = fmaxf(M1c, __shfl_xor_sync(FULL, M1c, 1));
+    M2c = fmaxf(M2c, __shfl_xor_sync(FULL, M2c, 1));
+  }
+  const int R1 = bitlen(M1), R2 = bitlen(M2), R1c = bitlen(M1c), R2c = bitlen(M2c);
 
-  // Tile costs (Eq. 3; variants 3 and 4 pay 4 bytes for mu): sums over the tile's 8 lanes
-  // of the block costs as 16-bit halves; centring changes block 0 only.
-  const uint32_t S1 = block_cost(R1), S2 = block_cost(R2);
-  uint32_t A = S1 | (S2 << 16);
-  uint32_t B = g == 0 ? (block_cost(R1c) | (block_cost(R2c) << 16)) : A;
+  // Tile costs (Eq. 3; variants 3 and 4 pay 4 bytes for mu): sums over the tile's lanes of
+  // the block costs as 16-bit halves.
+  uint32_t A = block_cost(R1) | (block_cost(R2) << 16);
+  uint32_t B = block_cost(R1c) | (block_cost(R2c) << 16);
 #pragma unroll
-  for (int o = 1; o <= 4; o <<= 1) {
+  for (int o = 1; o < LT; o <<= 1) {
     A += __shfl_xor_sync(FULL, A, o);
     B += __shfl_xor_sync(FULL, B, o);
   }
@@ -355,17 +368,17 @@ __device__ __forceinline__ void plan_quad(const float (&d)[32], const float r, c
   if (C4 < best) { v = 3; best = C4; }
   const bool second = (v & 1) != 0, centred = v >= 2;
 
-  int Rg = second ? R2 : R1;
-  if (g == 0 && centred) Rg = second ? R2c : R1c;
+  const int Rg = centred ? (second ? R2c : R1c) : (second ? R2 : R1);
   // Rate header (Sec. 3.1): block 0 carries bit 7 = order 2, bit 6 = centred.
-  if (live) {
+  if (live && (Cfg::kBlockLanes == 1 || (lane & 1) == 0)) {
     uint32_t hb = uint32_t(Rg);
     if (g == 0) hb |= (second ? 0x80u : 0u) | (centred ? 0x40u : 0u);
-    hdr[lane] = uint8_t(hb);
+    hdr[lane / Cfg::kBlockLanes] = uint8_t(hb);
   }
 
-  // Offsets: one scan over the quad's 32 blocks in stream order of the lane's bytes (its
-  // block's data, preceded in block 0 of a centred tile by the 4-byte mean).
+  // Offsets: one scan over the quad's 32 lanes in stream order of the lane's bytes (its
+  // block's data, preceded in block 0 of a centred tile by the 4-byte mean). The words of a
+  // 64-element block alternate between its lanes, starting where the first lane's bytes do.
   const bool slot = live && centred && g == 0;
   const uint32_t mine = live ? block_cost(Rg) + (slot ? 4u : 0u) : 0u;
   uint32_t inc = mine;
@@ -377,6 +390,7 @@ __device__ __forceinline__ void plan_quad(const float (&d)[32], const float r, c
   P.mu_off = excl;
   P.mu = mu;
   P.off = excl + (slot ? 4u : 0u);
+  if (Cfg::kBlockLanes == 2 && (lane & 1)) P.off = excl - mine + 4u;
   P.R = live ? Rg : 0;
   P.Rmax = int(__reduce_max_sync(FULL, live ? uint32_t(Rg) : 0u));
 
@@ -413,33 +427,37 @@ __device__ __forceinline__ void plan_quad(const float (&d)[32], const float r, c
 
 // Writes this lane's block words (sign map, then bit-planes from the least significant) at
 // the shared-memory address blk, for the quad's byte-slices that any lane needs.
+template <typename Cfg>
 __device__ __forceinline__ void encode_block(const QuadPlan& P, uint32_t blk) {
+  constexpr int W = Cfg::kWordBytes;
   uint32_t X[8];
   if (P.Rmax > 0) {
     if (P.R > 0) sts32(blk, P.signs);
     planes8<0>(P.v, X);
 #pragma unroll
     for (int b = 0; b < 8; ++b)
-      if (b < P.R) sts32(blk + 4 + 4 * b, X[b]);
+      if (b < P.R) sts32(blk + W * (1 + b), X[b]);
   }
   if (P.Rmax > 8) {
     planes8<1>(P.v, X);
 #pragma unroll
     for (int b = 0; b < 8; ++b)
-      if (8 + b < P.R) sts32(blk + 36 + 4 * b, X[b]);
+      if (8 + b < P.R) sts32(blk + W * (9 + b), X[b]);
   }
   if (P.Rmax > 16) {
     planes8<2>(P.v, X);
 #pragma unroll
     for (int b = 0; b < 8; ++b)
-      if (16 + b < P.R) sts32(blk + 68 + 4 * b, X[b]);
+      if (16 + b < P.R) sts32(blk + W * (17 + b), X[b]);
   }
 }
 
 // kGiven: the multipass evaluation's encoding pass (selection from a.given_costs).
 // kFeat: fields' switched-off features honoured; without it the full method is compiled
-// with none of that handling.
-template <bool kGiven, bool kFeat>
+// with none of that handling. Cfg: the tile configuration. (Every configuration through this
+// one kernel: a 256^3 field at 64 x 8 takes 46 us, where a cost pass, a scan of the tile sizes,
+// an encoding pass and a preamble kernel, with the field read twice, took 102 us.)
+template <bool kGiven, bool kFeat, typename Cfg>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(KernelArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   CompressSmem& S = *reinterpret_cast<CompressSmem*>(smem_raw);
@@ -497,18 +515,18 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
               FieldInfo* fi = single ? a.fields : a.fields + a.chunk_field[c];
               const uint64_t first = fi->chunk_first;
               const uint64_t lc = c - first;
-              const uint64_t tile0 = lc * kCChunkTiles;
-              const uint64_t e0 = tile0 * kTile;
+              const uint64_t tile0 = lc * Cfg::kChunkTiles;
+              const uint64_t e0 = lc * kCChunkElems;
               const uint64_t T = fi->T;
               ci.chunk = c;
               ci.in = fi->in + e0;
               ci.out = fi->out;
               ci.fi = fi;
               ci.tile0 = tile0;
-              ci.data_base = 64 + 8 * T;
+              ci.data_base = 64 + Cfg::kT * T;
               ci.cap = fi->cap;
               ci.chunk_first = first;
-              ci.ntiles = uint32_t(min(uint64_t(kCChunkTiles), T - tile0));
+              ci.ntiles = uint32_t(min(uint64_t(Cfg::kChunkTiles), T - tile0));
               ci.cnt = uint32_t(min(fi->n - e0, uint64_t(kCChunkElems)));
               ci.r = fi->r;
               ci.off = fi->features_off;
@@ -553,7 +571,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
                   }
                 }
               }
-              if (lane == 0 && (ci.flags & kInfoLast)) write_preamble(ci.fi, excl + tot);
+              if (lane == 0 && (ci.flags & kInfoLast)) write_preamble(ci.fi, excl + tot, Cfg::kT);
             }
           }
           // the runs are read: their ring space goes back to the compute warps
@@ -707,18 +725,19 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     }
     uint32_t qlen = 0;
     QuadPlan P;
-    const int qt0 = kQuadTiles * warp;            // the quad's first tile in the chunk
+    const int qt0 = Cfg::kQuadTiles * warp;            // the quad's first tile in the chunk
     const bool any = !end && (flags & kInfoOk) && qt0 < int(ci.ntiles);
     if (any) {
-      const int t = qt0 + (lane >> 3);
+      const int t = qt0 + lane / Cfg::kLanes;
       const bool live = t < int(ci.ntiles);
       const uint32_t foff = kFeat ? ci.off : 0u;
-      const bool restart = (lane & 7) == 0 || (foff & kOffCross);
+      const bool restart = lane % Cfg::kLanes == 0 ||
+                           ((foff & kOffCross) && lane % Cfg::kBlockLanes == 0);
       const int pen2 = (foff & kOffLz2) ? 0x10000 : 0;
       const int pen3 = (foff & kOffCenter) ? 0x10000 : 0;
-      uint8_t* hdr = ci.out + 64 + 8 * (ci.tile0 + uint64_t(qt0));
+      uint8_t* hdr = ci.out + 64 + Cfg::kT * (ci.tile0 + uint64_t(qt0));
       // (a lane of a missing tile reads the quad's first tile's given costs)
-      plan_quad<kGiven>(d, ci.r, lane, live, restart, pen2, pen3,
+      plan_quad<kGiven, Cfg>(d, ci.r, lane, live, restart, pen2, pen3,
                         a.given_costs + ci.tile0 + uint64_t(live ? t : qt0), a.given_T, hdr, P);
       qlen = P.qlen;
     }
@@ -790,7 +809,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     if (any && ok_run) {
       const uint32_t run = ring_u32 + pos;
       if (P.mu_slot) sts32(run + P.mu_off, __float_as_uint(P.mu));
-      encode_block(P, run + P.off);
+      encode_block<Cfg>(P, run + P.off);
     }
     if (lane == 0) {
       S.qpos[b][warp] = pos;
@@ -811,17 +830,22 @@ LaunchCfg compress_cfg() {
   return cache.get([] {
     LaunchCfg c;
     c.smem = int(sizeof(CompressSmem));
-    cudaFuncSetAttribute(fsz_compress_kernel<false, false>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
-    cudaFuncSetAttribute(fsz_compress_kernel<false, true>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
-    cudaFuncSetAttribute(fsz_compress_kernel<true, false>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
+    auto allow = [&](auto kernel) {
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
+    };
+    allow(fsz_compress_kernel<false, false, DefaultCfg>);
+    allow(fsz_compress_kernel<false, true, DefaultCfg>);
+    allow(fsz_compress_kernel<true, false, DefaultCfg>);
+    allow(fsz_compress_kernel<false, true, TileCfg<32, 4>>);
+    allow(fsz_compress_kernel<false, true, TileCfg<32, 16>>);
+    allow(fsz_compress_kernel<false, true, TileCfg<64, 4>>);
+    allow(fsz_compress_kernel<false, true, TileCfg<64, 8>>);
+    allow(fsz_compress_kernel<false, true, TileCfg<64, 16>>);
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fsz_compress_kernel<false, false>, kThreads,
-                                                  c.smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fsz_compress_kernel<false, false, DefaultCfg>,
+                                                  kThreads, c.smem);
     c.sms = sms;
     c.per = per > 0 ? per : 1;
     c.grid = sms * c.per;
@@ -829,19 +853,35 @@ LaunchCfg compress_cfg() {
   });
 }
 
-void launch_compress(const KernelArgs& args, uint64_t max_chunks, cudaStream_t st, CompressKind kind) {
+namespace {
+template <bool kGiven, bool kFeat, typename Cfg>
+void launch(const KernelArgs& args, uint64_t max_chunks, cudaStream_t st) {
   const LaunchCfg c = compress_cfg();
-  const int g = sched_grid(c, kSchedCompress, max_chunks);
   KernelArgs a = args;
   a.ticket_chunks = uint32_t(g_schedule.c_ticket_chunks);
   a.ticket_lead = uint32_t(g_schedule.c_ticket_lead);
   a.min_tickets = uint32_t(g_schedule.min_tickets);
+  launch_dependent(fsz_compress_kernel<kGiven, kFeat, Cfg>, sched_grid(c, kSchedCompress, max_chunks),
+                   kThreads, c.smem, st, a);
+}
+}  // namespace
+
+void launch_compress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st, CompressKind kind) {
   if (kind == kCompressFeatures)
-    launch_dependent(fsz_compress_kernel<false, true>, g, kThreads, c.smem, st, a);
+    launch<false, true, DefaultCfg>(a, max_chunks, st);
   else if (kind == kCompressGiven)
-    launch_dependent(fsz_compress_kernel<true, false>, g, kThreads, c.smem, st, a);
+    launch<true, false, DefaultCfg>(a, max_chunks, st);
   else
-    launch_dependent(fsz_compress_kernel<false, false>, g, kThreads, c.smem, st, a);
+    launch<false, false, DefaultCfg>(a, max_chunks, st);
+}
+
+void launch_compress_tiled(const KernelArgs& a, uint64_t max_chunks, int B, int T, cudaStream_t st) {
+  if (B == 32 && T == 4) launch<false, true, TileCfg<32, 4>>(a, max_chunks, st);
+  else if (B == 32 && T == 8) launch<false, true, DefaultCfg>(a, max_chunks, st);
+  else if (B == 32 && T == 16) launch<false, true, TileCfg<32, 16>>(a, max_chunks, st);
+  else if (B == 64 && T == 4) launch<false, true, TileCfg<64, 4>>(a, max_chunks, st);
+  else if (B == 64 && T == 8) launch<false, true, TileCfg<64, 8>>(a, max_chunks, st);
+  else launch<false, true, TileCfg<64, 16>>(a, max_chunks, st);
 }
 
 }  // namespace fsz

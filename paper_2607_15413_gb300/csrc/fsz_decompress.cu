@@ -34,11 +34,13 @@ constexpr int kThreads = (kDecodeWarps + 2) * 32;
 #endif
 constexpr int kMaxRecs = kMaxDecRecords;  // chunk records (fetched .. decoded): up to
 constexpr uint32_t kRingBytes = FSZ_DEC_RING_BYTES;  // payload byte ring
-constexpr int kQuadTiles = 4;  // tiles per decode warp and iteration
-// Ring bytes a chunk can take: its payload (at most kDChunkTiles header-valid tiles) from
-// the 16-byte boundary below its start, rounded up to 16 bytes.
-constexpr uint32_t kMaxChunkRingBytes = kDChunkTiles * kMaxDecTileBytes + 32;
-static_assert(kDChunkTiles <= 32, "one lane per tile in the chunk scan");
+constexpr int kQuadElems = 1024;  // elements per decode warp and chunk
+static_assert(kDecodeWarps * kQuadElems == kDChunkElems, "a chunk is one quad per decode warp");
+// Ring bytes a chunk can take: its payload (header-valid rates go up to 31: 128 bytes per 32
+// elements, and up to 64 means) from the 16-byte boundary below its start, rounded up to 16
+// bytes.
+constexpr uint32_t kMaxChunkRingBytes = kDChunkElems / 32 * 128 + 64 * 4 + 32;
+constexpr int kHdrUnits = 32;     // a chunk's rate bytes, 8 at a time (64-element blocks: 16)
 static_assert(kRingBytes % 16 == 0 && kRingBytes >= kMaxChunkRingBytes, "the ring holds the largest chunk");
 
 constexpr uint32_t kNoneChunk = 0xffffffffu;
@@ -50,15 +52,15 @@ constexpr uint32_t kNoneChunk = 0xffffffffu;
 // A chunk's header and parameters, from the header warp to the loader and the decode
 // warps through shared memory (keeps dependent global loads off the decode path).
 struct ChunkRec {
-  uint64_t hdr[kDChunkTiles];
-  uint64_t boff[kDChunkTiles];  // block word offsets of each tile (block_word_offsets)
-  uint32_t toff[kDChunkTiles];
+  uint64_t hdr[kHdrUnits];
+  uint64_t boff[kHdrUnits];  // block word offsets inside each unit (block_word_offsets)
+  uint32_t toff[kHdrUnits];  // byte offset of each unit's data in the payload
   FieldInfo* fi;
   float* dout;           // the chunk's first output element
   const uint8_t* sin;    // the field's stream
   uint64_t in_bytes;     // its size
   uint64_t data_bytes;   // tile data bytes the preamble declares
-  uint64_t data_base;    // 64 + 8T: start of the tile data
+  uint64_t data_base;    // start of the tile data, after the rate headers
   uint64_t excl;         // byte offset of the chunk's payload in the tile data
   uint32_t chunk;        // global chunk index, or kNoneChunk
   uint32_t last;         // the field's last chunk
@@ -74,7 +76,7 @@ struct ChunkRec {
 
 struct __align__(16) DecompressSmem {
   uint8_t ring[kRingBytes];
-  float out[kDecodeWarps][kQuadTiles * kTile];  // per-warp re-layout of a quad's floats
+  float out[kDecodeWarps][kQuadElems];  // per-warp re-layout of a quad's floats
   ChunkRec rec[kMaxRecs];
   uint32_t ring_end[kMaxRecs];  // loader only: ring position (mod 2^32) after each chunk's bytes
   // fetched: record in (header -> loader); full: payload in (loader -> decode warps);
@@ -84,7 +86,7 @@ struct __align__(16) DecompressSmem {
 // two CTAs per SM (228 KiB of shared memory, 1 KiB of it reserved per CTA)
 static_assert(sizeof(DecompressSmem) <= 113 * 1024, "shared memory of one CTA");
 
-// Word offsets of the 8 blocks inside the tile's data (after mu), one per byte: the
+// Word offsets of a unit's 8 blocks inside its data (means not counted), one per byte: the
 // exclusive byte-wise prefix sum of the blocks' word counts (rate + 1, or 0; <= 224).
 __device__ __forceinline__ uint64_t block_word_offsets(uint64_t h) {
   const uint64_t R = h & 0x1F1F1F1F1F1F1F1FULL;
@@ -92,8 +94,10 @@ __device__ __forceinline__ uint64_t block_word_offsets(uint64_t h) {
   return (W * 0x0101010101010101ULL) << 8;
 }
 
-__device__ __forceinline__ bool header_reserved_bits_set(uint64_t h) {
-  return (h & 0x20u) || (h & 0xE0E0E0E0E0E0E000ULL);
+// A byte that begins a tile reserves bit 5 (bits 7 and 6 are its flags), the others bits 5-7.
+__device__ __forceinline__ bool header_reserved_bits_set(uint64_t h, int T, uint64_t unit) {
+  const uint64_t flags = 3 * unit_centring_bits(T, unit);  // 0x40 and 0x80
+  return (h & (0xE0E0E0E0E0E0E0E0ULL & ~flags)) != 0;
 }
 
 // *p if `in`, else 0, read here: a plain load is moved down to its use by the compiler, past
@@ -169,13 +173,13 @@ __device__ __forceinline__ float4 lds128(uint32_t addr) {
   return v;
 }
 
-// Inclusive prefix sum over a tile of x[0..31] in each lane (the lane's block), the 8
-// lanes of a tile carrying block to block: the lane's own prefix, then the exclusive scan
-// of the blocks' totals over the tile's lanes, plus `add`. Without the carried state
-// (indep) each block restarts. Lanes with `apply` false keep x; every lane of the warp
-// must call this (the scan's shuffles take the full warp), and the 8 lanes of a tile
-// agree on `apply`, so the scan segments of applying tiles see only their own lanes.
-template <bool kAny>
+// Inclusive prefix sum over a tile of x[0..31] in each lane, a tile's lanes (8 by default)
+// carrying from one to the next: the lane's own prefix, then the exclusive scan of the lanes'
+// totals, plus `add`. Without the carried state (indep) each block restarts. Lanes with
+// `apply` false keep x; every lane of the warp must call this (the scan's shuffles take the
+// full warp), and the lanes of a tile agree on `apply`, so the scan segments of applying
+// tiles see only their own lanes.
+template <bool kAny, typename Cfg>
 __device__ __forceinline__ void tile_prefix(uint32_t (&x)[32], const uint32_t add, const bool indep,
                                             const bool apply) {
   // the lane's prefix as four independent 8-element runs (short dependency chains), the
@@ -193,9 +197,15 @@ __device__ __forceinline__ void tile_prefix(uint32_t (&x)[32], const uint32_t ad
   }
   uint32_t inc = tot;
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) inc = scan_step_up<8>(inc, o);
+  for (int o = 1; o < Cfg::kLanes; o <<= 1) inc = scan_step_up<Cfg::kLanes>(inc, o);
   uint32_t ex = inc - tot;
-  if (kAny && indep) ex = 0;
+  if (kAny && indep) {
+    ex = 0;
+    if constexpr (Cfg::kBlockLanes == 2) {  // a 64-element block's second lane follows its first
+      const uint32_t before = __shfl_up_sync(0xffffffffu, tot, 1);
+      if (threadIdx.x & 1) ex = before;
+    }
+  }
   ex += add;
   if (apply) {
     const uint32_t e[4] = {ex, ex + o1, ex + o2, ex + o3};
@@ -204,21 +214,19 @@ __device__ __forceinline__ void tile_prefix(uint32_t (&x)[32], const uint32_t ad
   }
 }
 
-// Decodes one quad (4 tiles) with one warp into o (lane L: block L & 7 of tile L >> 3).
-// h, boff: the lane's tile's header and block word offsets; tp: shared-memory address of
-// the tile's data; live: the tile exists. Returns false if a tile's mean slot is
-// malformed. kAny: the instance that also decodes streams without the cross-block state
-// (`indep`: every block restarts from zero predecessors).
-template <bool kAny>
-__device__ __forceinline__ bool decompress_quad(const uint64_t h, const uint64_t boff,
-                                                const uint32_t tp, const bool live, const float s,
-                                                const int lane, const bool indep, float (&o)[32]) {
+// Decodes one quad (1024 elements) with one warp into o, lane L elements 32 L .. 32 L + 31: a
+// block, or half of a 64-element one (whose lanes' words alternate). flags: the first rate
+// byte of the lane's tile; Rg: the rate of the lane's block; tp, blk: shared-memory addresses
+// of the tile's data and of the lane's first word; live: the tile exists. Returns false if a
+// tile's mean slot is malformed. kAny: the instance that also decodes streams without the
+// cross-block state (`indep`: every block restarts from zero predecessors).
+template <bool kAny, typename Cfg>
+__device__ __forceinline__ bool decompress_quad(const uint32_t flags, const int Rg, const uint32_t tp,
+                                                const uint32_t blk, const bool live, const float s,
+                                                const bool indep, float (&o)[32]) {
   constexpr uint32_t FULL = 0xffffffffu;
-  const int g = lane & 7;
-  const bool second = (h & 0x80u) != 0, centred = (h & 0x40u) != 0;
-  const int Rg = live ? int((h >> (8 * g)) & 31u) : 0;
-  // d2: block offsets by a byte-wise prefix sum (done by the header warp)
-  const uint32_t blk = tp + (centred ? 4u : 0u) + 4u * uint32_t((boff >> (8 * g)) & 0xFFu);
+  constexpr uint32_t W = Cfg::kWordBytes;
+  const bool second = (flags & 0x80u) != 0, centred = (flags & 0x40u) != 0;
   bool good = true;
   int mu = 0;
   if (live && centred) {
@@ -248,7 +256,7 @@ __device__ __forceinline__ bool decompress_quad(const uint64_t h, const uint64_t
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
           const int j = 8 * c + b;  // plane j of x: magnitude plane j is the block's word j + 1
-          const uint32_t M = j < Rg ? lds32(blk + 4u * uint32_t(j + 1)) : 0u;
+          const uint32_t M = j < Rg ? lds32(blk + W * uint32_t(j + 1)) : 0u;
           const uint32_t y = M ^ S;
           X[c][b] = y ^ carry;
           carry &= y;
@@ -297,8 +305,8 @@ __device__ __forceinline__ bool decompress_quad(const uint64_t h, const uint64_t
   // sum of the prefix sum (the first sum rebuilds the LZ1 residuals); then + mu. The
   // quad's tiles may differ in their predictor: the first sum runs on the whole warp and
   // applies to the LZ2 tiles only.
-  if (__any_sync(FULL, second)) tile_prefix<kAny>(x, 0u, indep, second);
-  tile_prefix<kAny>(x, uint32_t(mu), indep, true);
+  if (__any_sync(FULL, second)) tile_prefix<kAny, Cfg>(x, 0u, indep, second);
+  tile_prefix<kAny, Cfg>(x, uint32_t(mu), indep, true);
 #pragma unroll
   for (int i = 0; i < 32; ++i) o[i] = __fmul_rn(__int2float_rn(int(x[i])), s);
   return __all_sync(FULL, good);
@@ -324,6 +332,7 @@ __device__ __forceinline__ Field field_of_record(const FieldInfo* fi) {
 
 // The field of a one-field call, from the preamble as it stands: within the stream's buffer
 // and the output's capacity whatever it says.
+template <typename Cfg>
 __device__ __forceinline__ Field field_of_stream(const KernelArgs& a) {
   Field f = {};
   f.sin = a.sin;
@@ -333,7 +342,7 @@ __device__ __forceinline__ Field field_of_stream(const KernelArgs& a) {
   const uint4* p = reinterpret_cast<const uint4*>(a.sin);
   const uint4 w0 = p[0], w3 = p[3];
   f.n = min(uint64_t(w0.z) | (uint64_t(w0.w) << 32), a.cap_elems);
-  f.T = min((f.n + kTile - 1) / kTile, (a.in_bytes - 64) / 8);
+  f.T = min((f.n + Cfg::kElems - 1) / Cfg::kElems, (a.in_bytes - 64) / Cfg::kT);
   f.s = __uint_as_float(w3.x);
   f.features_off = w3.y;
   f.data_bytes = uint64_t(w3.z) | (uint64_t(w3.w) << 32);
@@ -343,8 +352,9 @@ __device__ __forceinline__ Field field_of_stream(const KernelArgs& a) {
 // kAny: also decodes streams without the cross-block state. kPrezero: the output already
 // holds zeros; tiles whose 8 blocks all have rate 0 and no mean (all +0.0) are neither
 // decoded nor written (the adaptive pre-zero of Sec. 3.1 for high compression ratios).
-template <bool kAny, bool kPrezero>
-__global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs a) {
+// Cfg: the tile configuration.
+template <bool kAny, bool kPrezero, typename Cfg>
+__device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
   DecompressSmem& S = *reinterpret_cast<DecompressSmem*>(smem_raw);
   constexpr uint32_t FULL = 0xffffffffu;
@@ -377,7 +387,7 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
     uint64_t total = 0;  // chunks of the launch
     uint64_t c0 = 0;     // the group's first chunk
     uint32_t group = 1;
-    uint64_t h[kMaxTicketChunks];  // the lane's tile's header in each chunk, 0 beyond the field
+    uint64_t h[kMaxTicketChunks];  // the lane's unit of rate bytes in each chunk, 0 beyond the field
     uint32_t nt = 0;               // lane g: tiles of chunk g, 0 if there is none
     uint32_t fidx = 0;             // lane g: chunk g's field
     // the end of the previous group: the chunk after it, its offset in its field
@@ -392,14 +402,16 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
         fidx = a.chunk_field[c];
         f = field_of_record(a.fields + fidx);
       }
-      const uint64_t t0 = (c - f.first) * kDChunkTiles;
-      nt = mine ? uint32_t(min(uint64_t(kDChunkTiles), f.T - t0)) : 0u;
-      const uint64_t hp = reinterpret_cast<uint64_t>(f.sin) + 64 + 8 * t0;
+      const uint64_t t0 = (c - f.first) * Cfg::kChunkTiles;
+      nt = mine ? uint32_t(min(uint64_t(Cfg::kChunkTiles), f.T - t0)) : 0u;
+      const uint64_t hp = reinterpret_cast<uint64_t>(f.sin) + 64 + Cfg::kT * t0;
 #pragma unroll
       for (int g = 0; g < kMaxTicketChunks; ++g) {
-        const uint64_t p = __shfl_sync(FULL, hp, g);
-        h[g] = ld_now(reinterpret_cast<const unsigned long long*>(p) + lane,
-                      uint32_t(lane) < __shfl_sync(FULL, nt, g));
+        const uint64_t p = __shfl_sync(FULL, hp, g) + 8 * lane;
+        const uint32_t end = Cfg::kT * __shfl_sync(FULL, nt, g);  // rate bytes of the chunk
+        h[g] = ld_now(reinterpret_cast<const void*>(p), 8u * lane + 8u <= end);
+        if (Cfg::kT == 4 && 8u * lane + 4u == end)  // an odd number of 4-block tiles
+          h[g] = __ldg(reinterpret_cast<const uint32_t*>(p));
       }
     };
     // d3: a CTA's chunks only go up, so the previous group ended in this one's field if it ended
@@ -412,8 +424,8 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
       // One field: its preamble and the headers of the CTA's first ticket (its own number) are
       // read under the set-up kernel, which does not write them; what the preamble says counts
       // only once that kernel's verdict (the control words' chunk count) is in.
-      f = field_of_stream(a);
-      total = (f.T + kDChunkTiles - 1) / kDChunkTiles;
+      f = field_of_stream<Cfg>(a);
+      total = (f.T + Cfg::kChunkTiles - 1) / Cfg::kChunkTiles;
       group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
       c0 = uint64_t(blockIdx.x) * group;
       fetch_headers();
@@ -443,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
       // d2: tile sizes and their scans, the chunks side by side
       uint32_t mine[kMaxTicketChunks], inc[kMaxTicketChunks], tot[kMaxTicketChunks];
 #pragma unroll
-      for (int g = 0; g < kMaxTicketChunks; ++g) inc[g] = mine[g] = tile_bytes_from_header(h[g]);
+      for (int g = 0; g < kMaxTicketChunks; ++g) inc[g] = mine[g] = unit_bytes(h[g], Cfg::kB, Cfg::kT, lane);
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1)
 #pragma unroll
@@ -452,8 +464,7 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
       // cross-block state are decoded by the kAny instance only
       const bool unsupported = !kAny && (f.features_off & kOffCross) && nt > 0;
       if (unsupported) set_error(a.ctrl, a.fields + fidx, FSZ_ERR_INVALID_ARG);
-      const uint32_t forbid = ((f.features_off & kOffLz2) ? 0x80u : 0u) |
-                              ((f.features_off & kOffCenter) ? 0x40u : 0u);
+      const uint32_t forbid = ((f.features_off & kOffLz2) ? 2u : 0u) | ((f.features_off & kOffCenter) ? 1u : 0u);
       uint32_t bad = unsupported ? 1u : 0u;
       uint32_t my_tot = 0;
       uint64_t excl = warp_sum_u64(range_lane_sum(part, part_rest)) +
@@ -463,8 +474,8 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
 #pragma unroll
       for (int g = 0; g < kMaxTicketChunks; ++g) {
         tot[g] = __shfl_sync(FULL, inc[g], 31);
-        const uint32_t fb = __shfl_sync(FULL, forbid, g);
-        const bool b = __any_sync(FULL, header_reserved_bits_set(h[g]) || (uint32_t(h[g]) & fb) != 0);
+        const uint64_t fb = __shfl_sync(FULL, forbid, g) * unit_centring_bits(Cfg::kT, lane);
+        const bool b = __any_sync(FULL, header_reserved_bits_set(h[g], Cfg::kT, lane) || (h[g] & fb) != 0);
         if ((starts >> g) & 1u) excl = 0;
         if (lane == g) {
           my_tot = tot[g];
@@ -488,20 +499,20 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
       }
       if (uint32_t(lane) < group) {
         ChunkRec& q = S.rec[my_r];
-        const uint64_t t0 = (c0 + lane - f.first) * kDChunkTiles;
+        const uint64_t lc = c0 + lane - f.first;
         q.chunk = nt > 0 ? uint32_t(c0 + lane) : kNoneChunk;
-        q.last = t0 + kDChunkTiles >= f.T ? 1u : 0u;
+        q.last = (lc + 1) * Cfg::kChunkTiles >= f.T ? 1u : 0u;
         q.tot = my_tot;
         q.bad = bad;
         q.fi = a.fields + fidx;
         q.sin = f.sin;
         q.in_bytes = f.in_bytes;
         q.data_bytes = f.data_bytes;
-        q.data_base = 64 + 8 * f.T;
+        q.data_base = 64 + Cfg::kT * f.T;
         q.excl = my_excl;
-        q.dout = f.dout + t0 * kTile;
+        q.dout = f.dout + lc * kDChunkElems;
         q.ntiles = nt;
-        q.cnt = uint32_t(min(f.n - t0 * kTile, uint64_t(kDChunkElems)));
+        q.cnt = uint32_t(min(f.n - lc * kDChunkElems, uint64_t(kDChunkElems)));
         q.step = f.s;
         q.indep = (f.features_off & kOffCross) ? 1u : 0u;
       }
@@ -625,18 +636,38 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
       const uint32_t cnt = st.cnt;
       float* dout = st.dout;
       const uint32_t pay = smem_u32(S.ring) + st.pay;
-      const int nquads = (ntiles + kQuadTiles - 1) / kQuadTiles;
-      for (int qd = warp; qd < nquads; qd += kDecodeWarps) {
-        const int t = kQuadTiles * qd + (lane >> 3);
-        const bool live = t < ntiles;
-        const uint64_t h = live ? st.hdr[t] : 0ull;
-        // a pre-zeroed output: a tile whose rates are all 0 and that has no mean is +0.0
-        // throughout, neither decoded nor written; a quad of such tiles is skipped
-        const bool write_tile = live && (!kPrezero || (h & 0x1F1F1F1F1F1F1F5FULL) != 0);
-        if (kPrezero && !__any_sync(FULL, write_tile)) continue;
+      const int t = Cfg::kQuadTiles * warp + lane / Cfg::kLanes;  // the lane's tile in the chunk
+      const bool live = t < ntiles;
+      // the lane's block: byte j of header unit u; the unit that begins its tile is uf
+      const int u = (Cfg::kB == 32 ? 4 * warp + (lane >> 3) : 2 * warp + (lane >> 4));
+      const int j = (Cfg::kB == 32 ? lane : lane >> 1) & 7;
+      const int uf = Cfg::kT == 16 ? u & ~1 : u;
+      const uint64_t h = live ? st.hdr[u] : 0ull;
+      const uint64_t hf = Cfg::kT == 16 ? (live ? st.hdr[uf] : 0ull) : h;
+      const uint32_t flags = uint32_t(Cfg::kT == 4 ? h >> (8 * (j & 4)) : hf) & 0xFFu;
+      // a pre-zeroed output: a tile whose rates are all 0 and that has no mean is +0.0
+      // throughout, neither decoded nor written; a quad of such tiles is skipped
+      const bool write_tile = live && (!kPrezero || (h & 0x1F1F1F1F1F1F1F5FULL) != 0);
+      const uint32_t tmask = __ballot_sync(FULL, write_tile);
+      if (tmask != 0) {
+        const uint64_t boff = live ? st.boff[u] : 0ull;
+        // d2: the unit's data, the means before the block in it, and the block's word offset
+        // (a byte-wise prefix sum by the header warp)
+        uint32_t blk = pay + (live ? st.toff[u] : 0u);
+        uint32_t tp = Cfg::kT == 16 ? pay + (live ? st.toff[uf] : 0u) : blk;
+        blk += Cfg::kWordBytes * uint32_t((boff >> (8 * j)) & 0xFFu) + 4u * uint32_t(lane % Cfg::kBlockLanes);
+        if (Cfg::kT == 4) {  // the unit's first tile's mean, then the second's
+          if (h & 0x40u) blk += 4u;
+          if (j & 4) {
+            tp += Cfg::kWordBytes * uint32_t((boff >> 32) & 0xFFu) + ((h & 0x40u) ? 4u : 0u);
+            if (flags & 0x40u) blk += 4u;
+          }
+        } else if (u == uf && (flags & 0x40u)) {
+          blk += 4u;  // (a 16-block tile's second unit starts after the mean)
+        }
         float o[32];
-        good &= decompress_quad<kAny>(h, live ? st.boff[t] : 0ull, pay + (live ? st.toff[t] : 0u),
-                                      live, step, lane, st.indep != 0, o);
+        good = decompress_quad<kAny, Cfg>(flags, live ? int((h >> (8 * j)) & 31u) : 0, tp, blk, live, step,
+                                          st.indep != 0, o);
         // re-layout: lane L's block goes to row L of the buffer, 16-byte piece k at column
         // k ^ (L & 7) (conflict-free); then each piece P = 32 j + lane, read back in order,
         // is stored to the output, the warp writing 512 consecutive bytes per store
@@ -645,10 +676,9 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
 #pragma unroll
         for (int k = 0; k < 8; ++k)
           sts128(row + ((uint32_t(k << 4)) ^ sw), make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]));
-        const uint32_t tmask = __ballot_sync(FULL, write_tile && (lane & 7) == 0);
         __syncwarp();
-        const uint32_t e0 = uint32_t(kQuadTiles * qd) * kTile;  // the quad's first element
-        if (tmask == 0x01010101u && e0 + kQuadTiles * kTile <= cnt) {
+        const uint32_t e0 = uint32_t(kQuadElems * warp);  // the quad's first element
+        if (tmask == FULL && e0 + kQuadElems <= cnt) {
           // every tile of the quad is written in full: no per-store guards
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -664,7 +694,7 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
             const uint32_t rw = P >> 3;
             const float4 val = lds128(obuf + rw * 128u + (((P & 7u) ^ (rw & 7u)) << 4));
             const uint32_t e = e0 + 4 * P;
-            if (!((tmask >> (8 * (rw >> 3))) & 1u)) continue;  // (a tile not written)
+            if (!((tmask >> rw) & 1u)) continue;  // (a tile not written)
             if (e + 4 <= cnt) {
               *reinterpret_cast<float4*>(dout + e) = val;
             } else {
@@ -685,6 +715,30 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs 
   }
 }
 
+template <bool kAny, bool kPrezero>
+__global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs a) {
+  decompress_cta<kAny, kPrezero, DefaultCfg>(a);
+}
+
+// Any tile configuration: the stream's own, from its preamble (a configuration that does not
+// exist is refused by the set-up kernel; this one then finds no chunks). One kernel that
+// branches once, because the host does not know the configuration: with one launch per
+// configuration, five of them returning at once, a scan of the tile sizes in three launches
+// and one warp per tile, a 256^3 field at 64 x 8 took 93 us; this takes 26 us with its set-up.
+__global__ void __launch_bounds__(kThreads, 2) fsz_decompress_tiled_kernel(KernelArgs a) {
+  int B = 32, T = 8;
+  if (a.in_bytes < 64 || !config_of(*reinterpret_cast<const uint32_t*>(a.sin + 52), &B, &T)) B = 32, T = 8;
+  if (B == 32) {
+    if (T == 4) decompress_cta<true, false, TileCfg<32, 4>>(a);
+    else if (T == 8) decompress_cta<true, false, TileCfg<32, 8>>(a);
+    else decompress_cta<true, false, TileCfg<32, 16>>(a);
+  } else {
+    if (T == 4) decompress_cta<true, false, TileCfg<64, 4>>(a);
+    else if (T == 8) decompress_cta<true, false, TileCfg<64, 8>>(a);
+    else decompress_cta<true, false, TileCfg<64, 16>>(a);
+  }
+}
+
 }  // namespace
 
 LaunchCfg decompress_cfg() {
@@ -692,12 +746,13 @@ LaunchCfg decompress_cfg() {
   return cache.get([] {
     LaunchCfg c;
     c.smem = int(sizeof(DecompressSmem));
-    cudaFuncSetAttribute(fsz_decompress_kernel<false, false>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
-    cudaFuncSetAttribute(fsz_decompress_kernel<true, false>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
-    cudaFuncSetAttribute(fsz_decompress_kernel<false, true>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
+    auto allow = [&](auto kernel) {
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
+    };
+    allow(fsz_decompress_kernel<false, false>);
+    allow(fsz_decompress_kernel<true, false>);
+    allow(fsz_decompress_kernel<false, true>);
+    allow(fsz_decompress_tiled_kernel);
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -710,20 +765,26 @@ LaunchCfg decompress_cfg() {
   });
 }
 
-void launch_decompress(const KernelArgs& args, uint64_t max_chunks, cudaStream_t st,
-                       DecompressKind kind) {
+namespace {
+void launch(void (*kernel)(KernelArgs), const KernelArgs& args, uint64_t max_chunks, cudaStream_t st) {
   const LaunchCfg c = decompress_cfg();
-  const int g = sched_grid(c, kSchedDecompress, max_chunks);
   KernelArgs a = args;
   a.ticket_chunks = uint32_t(g_schedule.d_ticket_chunks);
   a.records = uint32_t(g_schedule.d_records);
   a.min_tickets = uint32_t(g_schedule.min_tickets);
+  launch_dependent(kernel, sched_grid(c, kSchedDecompress, max_chunks), kThreads, c.smem, st, a);
+}
+}  // namespace
+
+void launch_decompress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st, DecompressKind kind) {
   if (kind == kDecompressAny)
-    launch_dependent(fsz_decompress_kernel<true, false>, g, kThreads, c.smem, st, a);
+    launch(fsz_decompress_kernel<true, false>, a, max_chunks, st);
   else if (kind == kDecompressPrezeroed)
-    launch_dependent(fsz_decompress_kernel<false, true>, g, kThreads, c.smem, st, a);
+    launch(fsz_decompress_kernel<false, true>, a, max_chunks, st);
+  else if (kind == kDecompressTiled)
+    launch(fsz_decompress_tiled_kernel, a, max_chunks, st);
   else
-    launch_dependent(fsz_decompress_kernel<false, false>, g, kThreads, c.smem, st, a);
+    launch(fsz_decompress_kernel<false, false>, a, max_chunks, st);
 }
 
 }  // namespace fsz

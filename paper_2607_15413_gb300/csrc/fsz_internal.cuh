@@ -90,6 +90,37 @@ struct alignas(16) FieldInfo {
   uint32_t features_off;  // method features switched off (kOff* bits; 0: the full method)
 };
 
+// A tile configuration (Sec. 6.5): kB elements per block, kT blocks per tile; 32 x 8 is the
+// default. In both kernels a lane holds 32 consecutive elements and a warp works on a quad
+// of 1024 elements at a time, whatever the configuration: kLanes lanes make a tile, one or
+// two a block, and a chunk is kDChunkElems elements, so work assignment, staging and
+// placement are the same for all.
+template <int B, int T>
+struct TileCfg {
+  static constexpr int kB = B, kT = T;
+  static constexpr int kElems = B * T;            // 128 .. 1024
+  static constexpr int kLanes = kElems / 32;      // lanes of a tile: 4, 8, 16 or 32
+  static constexpr int kBlockLanes = B / 32;      // lanes of a block: 1 or 2
+  static constexpr int kWordBytes = B / 8;        // a sign-map or plane word
+  static constexpr int kQuadTiles = 1024 / kElems;
+  static constexpr int kChunkTiles = kDChunkElems / kElems;
+  static constexpr int kHdrUnits = kDChunkElems / B / 8;  // a chunk's rate bytes, 8 at a time
+  static_assert((B == 32 || B == 64) && (T == 4 || T == 8 || T == 16), "Table 8's configurations");
+};
+using DefaultCfg = TileCfg<32, 8>;
+
+// The configuration as the method word of the preamble (byte 52) holds it in bits 8-15.
+__host__ __device__ __forceinline__ uint32_t tile_word_of(int B, int T) {
+  return (B == 64 ? 1u : 0u) << 8 | (T == 4 ? 1u : T == 16 ? 2u : 0u) << 12;
+}
+__host__ __device__ __forceinline__ bool config_of(uint32_t word, int* B, int* T) {
+  const uint32_t bc = (word >> 8) & 0xF, tc = (word >> 12) & 0xF;
+  if (bc > 1 || tc > 2 || (word & 0xFFFF00F8u)) return false;
+  *B = bc == 1 ? 64 : 32;
+  *T = tc == 1 ? 4 : tc == 2 ? 16 : 8;
+  return true;
+}
+
 // Features a compression may switch off, for the ablation of Sec. 6.4: the state carried
 // across block boundaries (off: every block restarts from zero predecessors), the centred
 // variants, the second-order variants. Centring is defined on the carried state (Eq. 4),
@@ -499,13 +530,22 @@ __device__ __forceinline__ uint64_t lookback(const uint64_t* flags, int64_t gchu
 
 // ------------------------------------------------------------------ rate headers
 
-// Bytes of a tile from its 8 header bytes: sum of S_b (Eq. 3) + 4 for a centred tile.
-__device__ __forceinline__ uint32_t tile_bytes_from_header(uint64_t h) {
+// The rate bytes of a chunk are handled 8 at a time (a unit): the 8 blocks of a default tile,
+// two 4-block tiles, or half of a 16-block one. `unit` is the unit's number in the field.
+
+// Bits 0x40 of the unit's bytes that begin a tile (its centring flags).
+__device__ __forceinline__ uint64_t unit_centring_bits(int T, uint64_t unit) {
+  return T == 4 ? 0x0000004000000040ULL : T == 16 && (unit & 1) ? 0ULL : 0x40ULL;
+}
+
+// Data bytes of a unit's blocks: the sum of S_b (Eq. 3: B / 8 bytes per word), and 4 for each
+// centred tile that begins in it.
+__device__ __forceinline__ uint32_t unit_bytes(uint64_t h, int B, int T, uint64_t unit) {
   const uint64_t R = h & 0x1F1F1F1F1F1F1F1FULL;
   const uint64_t W = R + (((R + 0x7F7F7F7F7F7F7F7FULL) & 0x8080808080808080ULL) >> 7);
   const uint32_t lo = uint32_t(W), hi = uint32_t(W >> 32);
   const uint32_t words = ((lo * 0x01010101u) >> 24) + ((hi * 0x01010101u) >> 24);
-  return 4u * words + ((h & 0x40u) ? 4u : 0u);
+  return uint32_t(B / 8) * words + 4u * uint32_t(__popcll(h & unit_centring_bits(T, unit)));
 }
 
 // ------------------------------------------------------------------ float keys
@@ -521,7 +561,8 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 
 // 64-byte preamble of this library's stream (little-endian; written once per field by the
 // CTA that finishes the field's last chunk), and the field's total size.
-__device__ __forceinline__ void write_preamble(FieldInfo* fi, uint64_t data_bytes) {
+// `tile_blocks`: rate bytes per tile.
+__device__ __forceinline__ void write_preamble(FieldInfo* fi, uint64_t data_bytes, int tile_blocks = 8) {
   uint32_t w[16];
   w[0] = 0x315A5346u;  // "FSZ1"
   w[1] = 1u | (fi->ndim << 16) | (fi->mode << 24);
@@ -537,13 +578,13 @@ __device__ __forceinline__ void write_preamble(FieldInfo* fi, uint64_t data_byte
   w[10] = uint32_t(eb);
   w[11] = uint32_t(eb >> 32);
   w[12] = __float_as_uint(fi->s);
-  w[13] = fi->features_off;
+  w[13] = fi->features_off;  // switched-off features and the tile configuration
   w[14] = uint32_t(data_bytes);
   w[15] = uint32_t(data_bytes >> 32);
   uint4* dst = reinterpret_cast<uint4*>(fi->out);
 #pragma unroll
   for (int k = 0; k < 4; ++k) dst[k] = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
-  const uint64_t total = 64 + 8 * fi->T + data_bytes;
+  const uint64_t total = 64 + uint64_t(tile_blocks) * fi->T + data_bytes;
   fi->data_bytes = data_bytes;
   if (fi->out_bytes) *fi->out_bytes = total;
 }
@@ -635,6 +676,8 @@ void launch_stats_batch(const KernelArgs& a, uint64_t max_chunks, cudaStream_t s
 // with switched-off features honoured per field (fsz_compress_features, batches); the
 // multipass evaluation's encoding pass (selection from a.given_costs).
 enum CompressKind { kCompressFull = 0, kCompressFeatures = 1, kCompressGiven = 2 };
+// A field in a tile configuration (its switched-off features honoured).
+void launch_compress_tiled(const KernelArgs& a, uint64_t max_chunks, int B, int T, cudaStream_t st);
 void launch_compress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st,
                      CompressKind kind = kCompressFull);
 // The multipass evaluation: one pass per variant writing its tile costs, then the
@@ -642,15 +685,18 @@ void launch_compress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st,
 void launch_cost_pass(const KernelArgs& a, int variant, uint32_t* costs, cudaStream_t st);
 
 // Decoder instances: the full method's; one that also decodes streams without the
-// cross-block state; one for a pre-zeroed output that skips all-zero tiles.
-enum DecompressKind { kDecompressFull = 0, kDecompressAny = 1, kDecompressPrezeroed = 2 };
+// cross-block state; one for a pre-zeroed output that skips all-zero tiles; one for streams of
+// any tile configuration.
+enum DecompressKind { kDecompressFull = 0, kDecompressAny = 1, kDecompressPrezeroed = 2, kDecompressTiled = 3 };
 void launch_decompress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st,
                        DecompressKind kind = kDecompressFull);
 // Single-field set-up: fills in the control words and the field record; for compression it
 // clears the lookback flags, for decompression it sizes the chunks' payloads (no memset of
 // the workspace needed). launch_sizes: the sizing of a planned batch.
 void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t chunk_cap, cudaStream_t st);
-void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st);
+// tiled: any tile configuration's stream (of at most max_chunks chunks).
+void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st,
+                             bool tiled = false);
 void launch_sizes(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st);
 void launch_plan_compress(const KernelArgs& a, const fsz_cfield* d_fields, uint32_t nfields,
                           uint64_t chunk_cap, cudaStream_t st);

@@ -262,6 +262,8 @@ __device__ uint32_t plan_cfield(FieldInfo* fi, const fsz_cfield& d) {
 
 // Parses and checks a stream's preamble (the same rules as the format's definition:
 // magic, version, ndim, mode, dims product, positive finite eb and step, sizes).
+// kTiled: streams of any tile configuration.
+template <bool kTiled>
 __device__ uint32_t plan_dfield(FieldInfo* fi, const uint8_t* in, uint64_t in_bytes, float* out,
                                 uint64_t cap_elems) {
   fi->sin = in;
@@ -298,13 +300,19 @@ __device__ uint32_t plan_dfield(FieldInfo* fi, const uint8_t* in, uint64_t in_by
   const float sv = __uint_as_float(w[12]);
   if (!(eb > 0.0) || isinf(eb)) return FSZ_ERR_CORRUPT;
   if (!(sv >= 1.5777218104420236e-30f) || isinf(sv)) return FSZ_ERR_CORRUPT;  // 2^-99
-  if (w[13] & 0xFF00u) return FSZ_ERR_INVALID_ARG;  // a tile configuration: fsz_decompress_tiled
-  if (!features_valid(w[13])) return FSZ_ERR_CORRUPT;
+  int B = 32, TB = 8;
+  if constexpr (kTiled) {
+    if (!config_of(w[13], &B, &TB) || !features_valid(w[13] & 7u)) return FSZ_ERR_CORRUPT;
+  } else {
+    if (w[13] & 0xFF00u) return FSZ_ERR_INVALID_ARG;  // a tile configuration: fsz_decompress_tiled
+    if (!features_valid(w[13])) return FSZ_ERR_CORRUPT;
+  }
   fi->features_off = w[13];
   const uint64_t db = uint64_t(w[14]) | (uint64_t(w[15]) << 32);
-  const uint64_t T = (n + kTile - 1) / kTile;
-  if (in_bytes - 64 < 8 * T) return FSZ_ERR_CORRUPT;
-  if (db > in_bytes - 64 - 8 * T) return FSZ_ERR_CORRUPT;
+  const uint32_t tile = uint32_t(B * TB);
+  const uint64_t T = (n + tile - 1) >> (31 - __clz(int(tile)));  // (a power of two)
+  if (in_bytes - 64 < TB * T) return FSZ_ERR_CORRUPT;
+  if (db > in_bytes - 64 - TB * T) return FSZ_ERR_CORRUPT;
   fi->n = n;
   fi->T = T;
   fi->ndim = ndim;
@@ -313,7 +321,7 @@ __device__ uint32_t plan_dfield(FieldInfo* fi, const uint8_t* in, uint64_t in_by
   fi->s = sv;
   fi->data_bytes = db;
   if (n > cap_elems) return FSZ_ERR_CAPACITY;
-  fi->nchunks = (T + kDChunkTiles - 1) / kDChunkTiles;
+  fi->nchunks = (n + kDChunkElems - 1) / kDChunkElems;
   return FSZ_OK;
 }
 
@@ -375,8 +383,8 @@ constexpr int kSizeWarps = 16;
 constexpr int kSizeThreads = 32 * kSizeWarps;
 constexpr int kChunksPerWarp = kSumBlock / kSizeWarps;  // of a block: warp, warp + kSizeWarps
 
-// Records the sizes of one block of chunks; bytes[k]: this lane's tile of chunk
-// kSumBlock * block + kSizeWarps * k + warp (0 beyond the last tile).
+// Records the sizes of one block of chunks; bytes[k]: this lane's unit of chunk
+// kSumBlock * block + kSizeWarps * k + warp (0 beyond the last one).
 __device__ __forceinline__ void write_chunk_sizes(const KernelArgs& a, uint64_t block, uint64_t total,
                                                   const uint32_t (&bytes)[kChunksPerWarp],
                                                   uint32_t* s_sum) {
@@ -402,8 +410,9 @@ __device__ __forceinline__ void write_chunk_sizes(const KernelArgs& a, uint64_t 
 // after it. The element count is read from the preamble as it stands, bounded by the
 // output's capacity, and the headers within the stream's buffer; the sizes of a stream that
 // the parsing refuses are not used.
-__global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(
-    KernelArgs a, uint64_t chunk_cap) {
+template <bool kTiled>
+__global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(KernelArgs a,
+                                                                            uint64_t chunk_cap) {
   const uint8_t* const in = a.sin;
   const uint64_t in_bytes = a.in_bytes, cap_elems = a.cap_elems;
   __shared__ uint32_t s_sum[kSumBlock];
@@ -412,19 +421,29 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(
   grid_release();
   const unsigned long long* const hdr = reinterpret_cast<const unsigned long long*>(in + 64);
   const uint64_t n = in_bytes >= 64 ? *reinterpret_cast<const uint64_t*>(in + 8) : 0;
-  const uint64_t readable = in_bytes >= 64 ? (in_bytes - 64) / 8 : 0;  // whole headers in the buffer
-  auto tile = [&](uint64_t b, int k) {
-    return (b * kSumBlock + kSizeWarps * k + warp) * kDChunkTiles + lane;
+  const uint64_t room = in_bytes >= 64 ? in_bytes - 64 : 0;  // bytes after the preamble
+  int B = 32, TB = 8;
+  if constexpr (kTiled) {
+    if (in_bytes >= 64 && !config_of(*reinterpret_cast<const uint32_t*>(in + 52), &B, &TB)) B = 32, TB = 8;
+  }
+  // rate bytes 8 (u + 0 .. 7), or as many of them as there are before `end`
+  auto load_unit = [&](uint64_t u, uint64_t end) -> uint64_t {
+    if (8 * u + 8 <= end) return __ldg(hdr + u);
+    if (kTiled && 8 * u + 4 <= end) return __ldg(reinterpret_cast<const uint32_t*>(hdr + u));
+    return 0;
+  };
+  const uint32_t units = uint32_t(kDChunkElems / 8) / uint32_t(B);  // of a chunk: 32 or 16
+  auto unit = [&](uint64_t b, int k) {
+    return (b * kSumBlock + kSizeWarps * k + warp) * units + lane;
   };
   uint64_t h[kChunksPerWarp];
+  if constexpr (!kTiled) {
 #pragma unroll
-  for (int k = 0; k < kChunksPerWarp; ++k) {  // (issued with n's load)
-    const uint64_t t = tile(blockIdx.x, k);
-    h[k] = t < readable ? __ldg(hdr + t) : 0;
+    for (int k = 0; k < kChunksPerWarp; ++k) h[k] = load_unit(unit(blockIdx.x, k), room);  // (issued with n's load)
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     FieldInfo f = {};
-    uint32_t st = plan_dfield(&f, in, in_bytes, a.dout, cap_elems);
+    uint32_t st = plan_dfield<kTiled>(&f, in, in_bytes, a.dout, cap_elems);
     if (st == FSZ_OK && f.nchunks > chunk_cap) st = FSZ_ERR_WORKSPACE;
     if (st != FSZ_OK) f.nchunks = 0;
     f.status = st;
@@ -435,15 +454,17 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(
     *a.fields = f;
     *a.ctrl = c;
   }
-  const uint64_t T = min((min(n, cap_elems) + kTile - 1) / kTile, readable);
-  const uint64_t total = (T + kDChunkTiles - 1) / kDChunkTiles;  // <= chunk_cap
+  const uint64_t nc = min(n, cap_elems);
+  const uint64_t total = (nc + kDChunkElems - 1) / kDChunkElems;  // <= chunk_cap
+  const uint64_t hdr_bytes = min(((nc + B * TB - 1) >> (31 - __clz(B * TB))) * TB, room);
   for (uint64_t b = blockIdx.x; b * kSumBlock < total; b += gridDim.x) {
     uint32_t bytes[kChunksPerWarp];
 #pragma unroll
     for (int k = 0; k < kChunksPerWarp; ++k) {
-      const uint64_t t = tile(b, k);
-      if (b != blockIdx.x) h[k] = t < T ? __ldg(hdr + t) : 0;
-      bytes[k] = t < T ? tile_bytes_from_header(h[k]) : 0u;
+      const uint64_t u = unit(b, k);
+      const bool mine = uint32_t(lane) < units && 8 * u < hdr_bytes;
+      if (kTiled || b != blockIdx.x) h[k] = mine ? load_unit(u, hdr_bytes) : 0;
+      bytes[k] = mine ? unit_bytes(h[k], B, TB, u) : 0u;
     }
     write_chunk_sizes(a, b, total, bytes, s_sum);
   }
@@ -466,8 +487,8 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_sizes_kernel(KernelArgs a) {
         const FieldInfo* fi = a.fields + a.chunk_field[c];
         const uint64_t t = (c - fi->chunk_first) * kDChunkTiles + lane;
         if (t < fi->T)
-          bytes[k] = tile_bytes_from_header(
-              __ldg(reinterpret_cast<const unsigned long long*>(fi->sin + 64) + t));
+          bytes[k] = unit_bytes(__ldg(reinterpret_cast<const unsigned long long*>(fi->sin + 64) + t),
+                                32, 8, t);
       }
     }
     write_chunk_sizes(a, b, total, bytes, s_sum);
@@ -519,7 +540,7 @@ __global__ void __launch_bounds__(kPlanThreads) fsz_plan_kernel(KernelArgs a, co
         st = plan_cfield(fi, static_cast<const fsz_cfield*>(d_fields)[f]);
       } else {
         const fsz_dfield d = static_cast<const fsz_dfield*>(d_fields)[f];
-        st = plan_dfield(fi, static_cast<const uint8_t*>(d.in), d.in_bytes, d.out, d.out_capacity_elems);
+        st = plan_dfield<false>(fi, static_cast<const uint8_t*>(d.in), d.in_bytes, d.out, d.out_capacity_elems);
       }
       if (st != FSZ_OK) {
         set_error(a.ctrl, fi, st);
@@ -614,8 +635,8 @@ void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t ch
   launch_dependent(fsz_setup_compress_kernel, setup_grid(nflags), kSetupThreads, 0, st, a, fi, nflags);
 }
 
-void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st) {
-  launch_dependent(fsz_setup_decompress_kernel,
+void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st, bool tiled) {
+  launch_dependent(tiled ? fsz_setup_decompress_kernel<true> : fsz_setup_decompress_kernel<false>,
                    sizes_grid((a.cap_elems + kDChunkElems - 1) / kDChunkElems), kSizeThreads, 0, st, a,
                    chunk_cap);
 }
