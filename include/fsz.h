@@ -280,7 +280,7 @@ fsz_status fsz_get_schedule_limits(uint32_t* stats_max, uint32_t* compress_max,
  * follows from the previous one (without a lookback in compression, Sec. 4.4). Compression takes
  * tickets up to `compress_ticket_lead` chunks (1-3) ahead of its compute warps;
  * decompression keeps up to `decompress_records` chunks (2 x ticket chunks .. 16) between
- * ticket and decode per CTA. A launch whose chunks would give fewer than
+ * ticket and decode per CTA (near a launch's end at most 6, by tickets of at most 2). A launch whose chunks would give fewer than
  * `min_tickets_per_cta` tickets per CTA (0-64) at the requested ticket size takes tickets
  * of fewer chunks (down to 1), so that small fields and small batches still spread over
  * every CTA; 0 keeps the requested size at every launch size. Defaults: CTAs 0 (as many

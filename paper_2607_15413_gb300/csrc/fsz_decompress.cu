@@ -49,6 +49,13 @@ constexpr uint32_t kNoneChunk = 0xffffffffu;
 // and the group's byte offset is summed once. A CTA holds `records` chunks
 // (2 x ticket_chunks .. kMaxRecs) between ticket and decode.
 
+// Near the launch's end (its last kTailChunks chunks per CTA) tickets are at most kTailTicket
+// chunks and a CTA holds at most kTailAhead: what one CTA has taken no other can, and with up
+// to 16 chunks (30 us) held each the CTAs finished far apart. 512^3: 112.6 us without, 109.8
+// from the last 8 chunks on, 106.9 from 16, 106.2 from 32; batch of 32 fields 69.7, 66.0, 66.5,
+// 67.6 us; with kTailAhead 4 or 8: 106.8, 108.9 and 67.9, 67.0 us.
+constexpr uint32_t kTailChunks = 16, kTailTicket = 2, kTailAhead = 6;
+
 // A chunk's header and parameters, from the header warp to the loader and the decode
 // warps through shared memory (keeps dependent global loads off the decode path).
 struct ChunkRec {
@@ -121,30 +128,33 @@ __device__ __forceinline__ uint32_t ld_now32(const uint32_t* p, bool in) {
   return v;
 }
 
-// The payload bytes of chunks lo .. hi - 1 are the sum over the warp of every lane's
-// range_lane_sum: the chunk sizes up to the first and from the last multiple of kSumBlock and
-// the block sums between, all loads independent. A CTA's tickets lie about one grid of
-// tickets apart, so a launch of 304 CTAs x 4 chunks reads 38 block sums and at most 62 sizes
-// per ticket; only a longer stretch needs the loop.
+// The payload bytes of chunks lo .. hi - 1 are range_total of what every lane fetched: the
+// chunk sizes up to the first and from the last multiple of kSumBlock and the block sums
+// between, all loads independent. A CTA's tickets lie about one grid of tickets apart, so a
+// launch of 304 CTAs x 4 chunks reads 38 block sums and at most 62 sizes per ticket; only a
+// longer stretch needs the loop.
 constexpr int kRangeParts = 4;
 __device__ __forceinline__ void range_fetch(const uint32_t* sums, const uint32_t* block_sums,
-                                            uint64_t lo, uint64_t hi, uint32_t (&part)[kRangeParts],
+                                            uint32_t lo, uint32_t hi, uint32_t (&part)[kRangeParts],
                                             uint64_t* rest) {
   static_assert(kSumBlock == 32, "one lane per chunk of a block");
-  const int lane = threadIdx.x & 31;
-  const uint64_t b0 = (lo + 31) / 32, b1 = hi / 32;  // whole blocks b0 .. b1 - 1
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t b0 = (lo + 31) / 32, b1 = hi / 32;  // whole blocks b0 .. b1 - 1
   const bool whole = b0 < b1;                        // (without one: at most 62 chunks)
-  const uint64_t k0 = lo + lane, k1 = (whole ? 32 * b1 : lo + 32) + lane;
+  const uint32_t k0 = lo + lane, k1 = (whole ? 32 * b1 : lo + 32) + lane;
   part[0] = ld_now32(sums + k0, k0 < (whole ? 32 * b0 : hi));
   part[1] = ld_now32(sums + k1, k1 < hi);
   part[2] = ld_now32(block_sums + b0 + lane, b0 + lane < b1);
   part[3] = ld_now32(block_sums + b0 + 32 + lane, b0 + 32 + lane < b1);
   uint64_t v = 0;
-  for (uint64_t b = b0 + 64 + lane; b < b1; b += 32) v += ld_now32(block_sums + b, true);
+  for (uint32_t b = b0 + 64 + lane; b < b1; b += 32) v += ld_now32(block_sums + b, true);
   *rest = v;
 }
-__device__ __forceinline__ uint64_t range_lane_sum(const uint32_t (&part)[kRangeParts], uint64_t rest) {
-  return rest + part[0] + part[1] + part[2] + part[3];  // (each below 2^22)
+__device__ __forceinline__ uint64_t range_total(const uint32_t (&part)[kRangeParts], uint64_t rest) {
+  // at most 62 chunks and 64 blocks of 32: below 2^27 bytes
+  uint64_t v = __reduce_add_sync(0xffffffffu, part[0] + part[1] + part[2] + part[3]);
+  if (__any_sync(0xffffffffu, rest != 0)) v += warp_sum_u64(rest);
+  return v;
 }
 
 // Byte permute with the generic mode's sign replication (a selector nibble with bit 3 set
@@ -379,45 +389,64 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
     // A ticket is a group of up to kMaxTicketChunks consecutive chunks; lane g keeps and writes
     // what concerns chunk g as a whole, all lanes its tiles (lane = tile), the chunks side by
     // side. This warp feeds all the others and shares their issue slots: with the chunks one
-    // after another and a ticket's atomic and loads in line it was the slowest stage. Whole
-    // calls before and after: 512^3 118.5 and 112.9 us, 16 M particles 29.5 and 24.6 us, batch
-    // of 32 fields 75.7 and 70.1 us.
+    // after another and a ticket's atomic and loads in line it was the slowest stage, and still
+    // was for launches of 1-chunk tickets (3 us each) until the scans were packed two to a
+    // register and the rest trimmed. Whole calls, at first / chunks side by side / trimmed:
+    // 512^3 118.5, 113.8, 112.6 us; 16 M particles 29.5, 25.1, 22.1 us; batch of 32 fields
+    // 75.7, 70.0, 69.7 us.
+    // (chunk numbers fit 32 bits: at most 2^27 and one per field)
     const bool single = a.sin != nullptr;
     Field f = {};        // lane g: chunk g's field (one field: the same in every lane)
-    uint64_t total = 0;  // chunks of the launch
-    uint64_t c0 = 0;     // the group's first chunk
+    uint32_t total = 0;  // chunks of the launch
+    uint32_t c0 = 0;     // the group's first chunk
     uint32_t group = 1;
     uint64_t h[kMaxTicketChunks];  // the lane's unit of rate bytes in each chunk, 0 beyond the field
     uint32_t nt = 0;               // lane g: tiles of chunk g, 0 if there is none
     uint32_t fidx = 0;             // lane g: chunk g's field
     // the end of the previous group: the chunk after it, its offset in its field
-    uint64_t prev_end = 0, prev_excl = 0;
-    uint64_t from = 0;   // the group's offset is counted from here: the field's start or prev_end
+    uint32_t prev_end = 0;
+    uint64_t prev_excl = 0;
+    uint32_t first0 = 0;  // the first chunk of the group's first field
     uint32_t part[kRangeParts];
     uint64_t part_rest = 0;
+    // Tickets 0 .. nbig - 1 are `full` chunks, the launch's last ones at most kTailTicket.
+    uint32_t full = 1, nbig = 0;
+    auto launch_tickets = [&]() {
+      full = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
+      nbig = total > gridDim.x * kTailChunks ? (total - gridDim.x * kTailChunks) / full : 0;
+    };
+    auto place = [&](uint32_t t) {
+      const bool big = t < nbig;
+      group = big ? full : min(full, kTailTicket);
+      c0 = big ? t * full : nbig * full + (t - nbig) * group;
+    };
     auto fetch_headers = [&]() {
-      const uint64_t c = c0 + lane;
+      const uint32_t c = c0 + lane;
       const bool mine = uint32_t(lane) < group && c < total;
       if (!single && mine) {
         fidx = a.chunk_field[c];
         f = field_of_record(a.fields + fidx);
       }
-      const uint64_t t0 = (c - f.first) * Cfg::kChunkTiles;
+      const uint64_t t0 = uint64_t(c - uint32_t(f.first)) * Cfg::kChunkTiles;
       nt = mine ? uint32_t(min(uint64_t(Cfg::kChunkTiles), f.T - t0)) : 0u;
       const uint64_t hp = reinterpret_cast<uint64_t>(f.sin) + 64 + Cfg::kT * t0;
 #pragma unroll
       for (int g = 0; g < kMaxTicketChunks; ++g) {
-        const uint64_t p = __shfl_sync(FULL, hp, g) + 8 * lane;
-        const uint32_t end = Cfg::kT * __shfl_sync(FULL, nt, g);  // rate bytes of the chunk
-        h[g] = ld_now(reinterpret_cast<const void*>(p), 8u * lane + 8u <= end);
-        if (Cfg::kT == 4 && 8u * lane + 4u == end)  // an odd number of 4-block tiles
-          h[g] = __ldg(reinterpret_cast<const uint32_t*>(p));
+        h[g] = 0;
+        if (uint32_t(g) < group) {
+          const uint64_t p = __shfl_sync(FULL, hp, g) + 8 * lane;
+          const uint32_t end = Cfg::kT * __shfl_sync(FULL, nt, g);  // rate bytes of the chunk
+          h[g] = ld_now(reinterpret_cast<const void*>(p), 8u * lane + 8u <= end);
+          if (Cfg::kT == 4 && 8u * lane + 4u == end)  // an odd number of 4-block tiles
+            h[g] = __ldg(reinterpret_cast<const uint32_t*>(p));
+        }
       }
     };
     // d3: a CTA's chunks only go up, so the previous group ended in this one's field if it ended
-    // behind the field's first chunk
+    // behind the field's first chunk: the offset counts from there, or from the field's start
     auto fetch_sizes = [&]() {
-      from = max(prev_end, __shfl_sync(FULL, f.first, 0));
+      first0 = __shfl_sync(FULL, uint32_t(f.first), 0);
+      const uint32_t from = max(prev_end, first0);
       range_fetch(a.sums, a.block_sums, from, c0 < total ? c0 : from, part, &part_rest);
     };
     if (single) {
@@ -425,85 +454,104 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
       // read under the set-up kernel, which does not write them; what the preamble says counts
       // only once that kernel's verdict (the control words' chunk count) is in.
       f = field_of_stream<Cfg>(a);
-      total = (f.T + Cfg::kChunkTiles - 1) / Cfg::kChunkTiles;
-      group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
-      c0 = uint64_t(blockIdx.x) * group;
+      total = uint32_t((f.T + Cfg::kChunkTiles - 1) / Cfg::kChunkTiles);
+      launch_tickets();
+      place(blockIdx.x);
       fetch_headers();
     }
     grid_wait();
     cta_sync();
-    const uint64_t verdict = a.ctrl->total_chunks;
+    const uint32_t verdict = uint32_t(a.ctrl->total_chunks);
     if (!single) {
       total = verdict;
-      group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
-      c0 = uint64_t(blockIdx.x) * group;
+      launch_tickets();
+      place(blockIdx.x);
       fetch_headers();
     }
     fetch_sizes();
     if (verdict == 0) nt = 0;
     total = verdict;
-    for (uint32_t seq = 0;; seq += group) {
+    const uint32_t off_bits = ((f.features_off & kOffLz2) ? 2u : 0u) | ((f.features_off & kOffCenter) ? 1u : 0u);
+    uint32_t r0 = 0;  // the group's first record: seq % recs
+    for (uint32_t seq = 0;;) {
       uint32_t next = 0;
       if (lane == 0) next = gridDim.x + atomicAdd(&a.ctrl->ticket, 1u);
       // the group's records must be free: their previous chunks decoded (the decode warps
       // finish chunks in order, so the last record's tells)
       const uint32_t sl = seq + group - 1;
-      if (sl >= recs && !mbar_wait(&S.done[sl % recs], ((sl / recs) - 1) & 1u, wait_ns)) {
-        if (lane == 0) set_error(a.ctrl, nullptr, FSZ_ERR_TIMEOUT);
-        return;
+      const uint32_t ahead = c0 < nbig * full ? recs : min(recs, kTailAhead);
+      if (sl >= ahead) {
+        const uint32_t w = sl - ahead;
+        if (!mbar_wait(&S.done[w % recs], (w / recs) & 1u, wait_ns)) {
+          if (lane == 0) set_error(a.ctrl, nullptr, FSZ_ERR_TIMEOUT);
+          return;
+        }
       }
-      // d2: tile sizes and their scans, the chunks side by side
-      uint32_t mine[kMaxTicketChunks], inc[kMaxTicketChunks], tot[kMaxTicketChunks];
+      // d2: sizes and their scans, two chunks to a register (a chunk is below 2^16 bytes)
+      uint32_t mine[kMaxTicketChunks], inc[kMaxTicketChunks / 2];
 #pragma unroll
-      for (int g = 0; g < kMaxTicketChunks; ++g) inc[g] = mine[g] = unit_bytes(h[g], Cfg::kB, Cfg::kT, lane);
+      for (int k = 0; k < kMaxTicketChunks / 2; ++k) {
+        mine[2 * k] = unit_bytes(h[2 * k], Cfg::kB, Cfg::kT, lane);
+        mine[2 * k + 1] = unit_bytes(h[2 * k + 1], Cfg::kB, Cfg::kT, lane);
+        inc[k] = mine[2 * k] | (mine[2 * k + 1] << 16);
+      }
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1)
 #pragma unroll
-        for (int g = 0; g < kMaxTicketChunks; ++g) inc[g] = scan_step_up<32>(inc[g], o);
+        for (int k = 0; k < kMaxTicketChunks / 2; ++k) inc[k] = scan_step_up<32>(inc[k], o);
       // a tile may not use a feature the stream has switched off; streams without the
       // cross-block state are decoded by the kAny instance only
       const bool unsupported = !kAny && (f.features_off & kOffCross) && nt > 0;
       if (unsupported) set_error(a.ctrl, a.fields + fidx, FSZ_ERR_INVALID_ARG);
-      const uint32_t forbid = ((f.features_off & kOffLz2) ? 2u : 0u) | ((f.features_off & kOffCenter) ? 1u : 0u);
-      uint32_t bad = unsupported ? 1u : 0u;
-      uint32_t my_tot = 0;
-      uint64_t excl = warp_sum_u64(range_lane_sum(part, part_rest)) +
-                      (prev_end > __shfl_sync(FULL, f.first, 0) ? prev_excl : 0);
-      uint64_t my_excl = 0;
-      const uint32_t starts = __ballot_sync(FULL, c0 + lane == f.first);  // bit g: a field's first chunk
+      const uint32_t forbid =
+          single ? off_bits
+                 : ((f.features_off & kOffLz2) ? 2u : 0u) | ((f.features_off & kOffCenter) ? 1u : 0u);
+      const bool any_forbid = __any_sync(FULL, forbid != 0);
+      uint32_t bad = 0;
 #pragma unroll
       for (int g = 0; g < kMaxTicketChunks; ++g) {
-        tot[g] = __shfl_sync(FULL, inc[g], 31);
-        const uint64_t fb = __shfl_sync(FULL, forbid, g) * unit_centring_bits(Cfg::kT, lane);
-        const bool b = __any_sync(FULL, header_reserved_bits_set(h[g], Cfg::kT, lane) || (h[g] & fb) != 0);
+        uint64_t not_allowed = 0;
+        if (any_forbid) not_allowed = __shfl_sync(FULL, forbid, g) * unit_centring_bits(Cfg::kT, lane);
+        if (header_reserved_bits_set(h[g], Cfg::kT, lane) || (h[g] & not_allowed) != 0) bad |= 1u << g;
+      }
+      bad = __reduce_or_sync(FULL, bad);
+      // offsets: each chunk follows from its predecessor, or starts its field
+      const uint32_t starts = __ballot_sync(FULL, c0 + lane == uint32_t(f.first));
+      uint64_t excl = range_total(part, part_rest) + (prev_end > first0 ? prev_excl : 0);
+      uint64_t my_excl = 0;
+      uint32_t my_tot = 0;
+      const uint32_t last[2] = {__shfl_sync(FULL, inc[0], 31), __shfl_sync(FULL, inc[1], 31)};
+#pragma unroll
+      for (int g = 0; g < kMaxTicketChunks; ++g) {
+        const uint32_t tot = (last[g / 2] >> (16 * (g & 1))) & 0xffffu;
         if ((starts >> g) & 1u) excl = 0;
         if (lane == g) {
-          my_tot = tot[g];
+          my_tot = tot;
           my_excl = excl;
-          if (b) bad = 1u;
         }
-        if (uint32_t(g) < group) excl += tot[g];
+        if (uint32_t(g) < group) excl += tot;
       }
       // the records
-      uint32_t r = seq % recs, my_r = 0;
+      uint32_t r = r0, my_r = 0;
 #pragma unroll
       for (int g = 0; g < kMaxTicketChunks; ++g) {
         if (uint32_t(g) < group) {
           ChunkRec& q = S.rec[r];
           q.hdr[lane] = h[g];
           q.boff[lane] = block_word_offsets(h[g]);
-          q.toff[lane] = inc[g] - mine[g];
+          q.toff[lane] = ((inc[g / 2] >> (16 * (g & 1))) & 0xffffu) - mine[g];
           if (lane == g) my_r = r;
           if (++r == recs) r = 0;
         }
       }
+      r0 = r;
       if (uint32_t(lane) < group) {
         ChunkRec& q = S.rec[my_r];
-        const uint64_t lc = c0 + lane - f.first;
-        q.chunk = nt > 0 ? uint32_t(c0 + lane) : kNoneChunk;
+        const uint64_t lc = c0 + lane - uint32_t(f.first);
+        q.chunk = nt > 0 ? c0 + lane : kNoneChunk;
         q.last = (lc + 1) * Cfg::kChunkTiles >= f.T ? 1u : 0u;
         q.tot = my_tot;
-        q.bad = bad;
+        q.bad = unsupported ? 1u : (bad >> lane) & 1u;
         q.fi = a.fields + fidx;
         q.sin = f.sin;
         q.in_bytes = f.in_bytes;
@@ -520,12 +568,13 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
       // (test hook: the record of skip_chunk is never handed over, nor any after it)
       const bool held = a.skip_chunk >= c0 && a.skip_chunk <= c0 + lane;
       // ... and after the launch's last chunk one record says that there are no more
-      const uint32_t live = total > c0 ? uint32_t(min(total - c0, uint64_t(group))) : 0u;
+      const uint32_t live = total > c0 ? min(total - c0, group) : 0u;
       if (uint32_t(lane) < group && !held && uint32_t(lane) <= live) mbar_arrive(&S.fetched[my_r]);
       if (c0 + group > total || __any_sync(FULL, uint32_t(lane) < group && held)) return;
       prev_end = c0 + group;
       prev_excl = excl;
-      c0 = uint64_t(__shfl_sync(FULL, next, 0)) * group;
+      seq += group;
+      place(__shfl_sync(FULL, next, 0));
       fetch_headers();
       fetch_sizes();
     }

@@ -11,8 +11,9 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 CHUNK = 8192
-# chunks: around one block, two blocks, and the ticket sizes 1-4 of a small and a large launch
-CHUNKS = [1, 2, 5, 31, 32, 33, 63, 64, 65, 97]
+# chunks: around one block, two blocks, the ticket sizes 1-4 of a small and a large launch, and
+# a field long enough that few CTAs reach the smaller tickets of a launch's end
+CHUNKS = [1, 2, 5, 31, 32, 33, 63, 64, 65, 97, 700]
 
 
 def _cuda():
@@ -37,7 +38,8 @@ def test_offsets_at_block_edges(fszlib, oracle, off):
     dev_streams = [torch.from_numpy(np.frombuffer(r, np.uint8).copy()).to(dev) for r in refs]
     scheds = [None, dict(decompress_ticket_chunks=4, decompress_records=8, min_tickets_per_cta=0),
               dict(decompress_ctas_per_sm=1, decompress_ticket_chunks=3, decompress_records=6,
-                   min_tickets_per_cta=0)]
+                   min_tickets_per_cta=0),
+              dict(decompress_ticket_chunks=1, decompress_records=2, min_tickets_per_cta=0)]
     try:
         for sched in scheds:
             assert fszlib.fsz_set_schedule_ex(sched) == fszlib.OK
@@ -50,6 +52,30 @@ def test_offsets_at_block_edges(fszlib, oracle, off):
                 assert np.array_equal(b.output(i).cpu().numpy().view(np.uint32), w)
     finally:
         fszlib.fsz_set_schedule_ex(None)
+
+
+@pytest.mark.parametrize("ticket,records", [(4, 16), (4, 9), (3, 7), (2, 4), (1, 16)])
+def test_tickets_from_the_first_to_the_tail(fszlib, ticket, records):
+    """Chunk counts around the point where a launch's tickets become smaller, against the
+    default schedule's reconstruction."""
+    dev = _cuda()
+    ctas = fszlib.fsz_get_schedule_limits()["sms"]     # one CTA per SM
+    for chunks in (16 * ctas - 1, 16 * ctas, 16 * ctas + 1, 16 * ctas + ticket + 1, 21 * ctas + 3):
+        n = chunks * CHUNK - 77
+        x = inputs.grf((n,), 7, "cuda")
+        s = fszlib.compress(x, 1e-3, fszlib.EB_REL)[0]
+        want = fszlib.decompress(s, n=n).clone()
+        try:
+            assert fszlib.fsz_set_schedule_ex(dict(decompress_ctas_per_sm=1, decompress_ticket_chunks=ticket,
+                                                   decompress_records=records, min_tickets_per_cta=0)) == fszlib.OK
+            out = torch.zeros(n, dtype=torch.float32, device=dev)
+            got = fszlib.decompress(s, n=n, out=out)
+        finally:
+            fszlib.fsz_set_schedule_ex(None)
+        assert torch.equal(got, want)
+        eb = fszlib.fsz_read_header(s[:64].cpu().numpy().tobytes())
+        err = (x.reshape(-1).double() - got.double()).abs().max().item()
+        assert err <= 1e-3 * (x.max() - x.min()).item() * (1 + 1e-6) and eb["n"] == n
 
 
 def test_offsets_with_two_calls_at_once(fszlib):
