@@ -132,6 +132,22 @@ fsz_status prepare_one(const float* d_in, fsz_dims dims, fsz_eb_mode mode, doubl
   return launched();
 }
 
+// The compression kernel behind prepare_one. `early`: right behind it, with nothing in
+// between that could write the input, so the kernel may read ahead under the value-range pass.
+fsz_status encode_one(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double eb,
+                      uint32_t features_off, void* d_out, uint64_t out_capacity, void* d_ws,
+                      uint64_t ws_bytes, fsz_stream stream, bool early) {
+  CompressCall call;
+  fsz_status st = check_compress(d_in, dims, mode, eb, d_out, out_capacity, d_ws, ws_bytes, &call,
+                                 features_off);
+  if (st != FSZ_OK || call.desc.nchunks == 0) return st;
+  KernelArgs a = make_args(d_ws, call.L);
+  a.early = early;
+  launch_compress(a, call.desc.nchunks, reinterpret_cast<cudaStream_t>(stream),
+                  features_off == 0 ? kCompressFull : kCompressFeatures);
+  return launched();
+}
+
 // One stream's decompression with the given decoder instance.
 fsz_status decompress_one(const void* d_in, uint64_t in_bytes, float* d_out,
                           uint64_t out_capacity_elems, void* d_ws, uint64_t ws_bytes,
@@ -204,23 +220,14 @@ fsz_status fsz_compress_encode(const float* d_in, fsz_dims dims, fsz_eb_mode mod
                                void* d_out, uint64_t out_capacity, uint64_t* d_out_bytes,
                                void* d_ws, uint64_t ws_bytes, fsz_stream stream) {
   (void)d_out_bytes;
-  CompressCall call;
-  fsz_status st = check_compress(d_in, dims, mode, eb, d_out, out_capacity, d_ws, ws_bytes, &call);
-  if (st != FSZ_OK) return st;
-  if (call.desc.nchunks == 0) return FSZ_OK;
-  launch_compress(make_args(d_ws, call.L), call.desc.nchunks, reinterpret_cast<cudaStream_t>(stream),
-                  kCompressFull);
-  return launched();
+  return encode_one(d_in, dims, mode, eb, 0, d_out, out_capacity, d_ws, ws_bytes, stream, false);
 }
 
 fsz_status fsz_compress(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double eb, void* d_out,
                         uint64_t out_capacity, uint64_t* d_out_bytes, void* d_ws, uint64_t ws_bytes,
                         fsz_stream stream) {
-  fsz_status st = fsz_compress_prepare(d_in, dims, mode, eb, d_out, out_capacity, d_out_bytes, d_ws,
-                                       ws_bytes, stream);
-  if (st != FSZ_OK) return st;
-  return fsz_compress_encode(d_in, dims, mode, eb, d_out, out_capacity, d_out_bytes, d_ws, ws_bytes,
-                             stream);
+  return fsz_compress_features(d_in, dims, mode, eb, 0, d_out, out_capacity, d_out_bytes, d_ws, ws_bytes,
+                               stream);
 }
 
 fsz_status fsz_compress_features(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double eb,
@@ -229,16 +236,8 @@ fsz_status fsz_compress_features(const float* d_in, fsz_dims dims, fsz_eb_mode m
                                  fsz_stream stream) {
   fsz_status st = prepare_one(d_in, dims, mode, eb, features_off, d_out, out_capacity, d_out_bytes,
                               d_ws, ws_bytes, stream);
-  if (st != FSZ_OK || features_off == 0)
-    return st != FSZ_OK ? st
-                        : fsz_compress_encode(d_in, dims, mode, eb, d_out, out_capacity, d_out_bytes,
-                                              d_ws, ws_bytes, stream);
-  CompressCall call;
-  st = check_compress(d_in, dims, mode, eb, d_out, out_capacity, d_ws, ws_bytes, &call, features_off);
-  if (st != FSZ_OK || call.desc.nchunks == 0) return st;
-  launch_compress(make_args(d_ws, call.L), call.desc.nchunks, reinterpret_cast<cudaStream_t>(stream),
-                  kCompressFeatures);
-  return launched();
+  if (st != FSZ_OK) return st;
+  return encode_one(d_in, dims, mode, eb, features_off, d_out, out_capacity, d_ws, ws_bytes, stream, true);
 }
 
 fsz_status fsz_compress_multipass(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double eb,
@@ -326,7 +325,8 @@ fsz_status fsz_compress_tiled(const float* d_in, fsz_dims dims, fsz_eb_mode mode
   call.desc.T = NT;
   call.desc.features_off = features_off | tile_word_of(int(block), int(tile_blocks));
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const KernelArgs a = make_args(d_ws, call.L);
+  KernelArgs a = make_args(d_ws, call.L);
+  a.early = true;
   launch_setup_compress(a, call.desc, call.L.chunk_cap, s);
   launch_stats(a, d_in, n, s);
   launch_compress_tiled(a, call.desc.nchunks, int(block), int(tile_blocks), s);

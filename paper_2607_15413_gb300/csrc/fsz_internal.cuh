@@ -169,6 +169,7 @@ struct KernelArgs {
   uint64_t* flags;       // compression: lookback flags
   uint32_t* sums;        // decompression: payload bytes of each chunk,
   uint32_t* block_sums;  // ... and of each kSumBlock consecutive ones
+  bool early = false;   // compression of one field: start under the value-range pass
   uint64_t skip_chunk;  // test hook: this chunk publishes no flag (decompression: no record)
   uint64_t timeout_ns;  // bound on every spin-wait
   // multipass compression only: the four variants' tile costs, variant-major (given_T
@@ -210,12 +211,12 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // a kernel's launch, its set-up and its loads of what no earlier kernel of the call writes
 // run under the predecessor's end. grid_wait() then holds it until the predecessor has
 // completed and its writes are visible; every kernel calls it, so completion stays in
-// stream order. grid_release() lets the successor's CTAs start. Only the set-up and
-// planning kernels call it, after grid_wait(), which also orders the successor's early
-// loads after everything before the call. The large kernels do not: a set-up CTA resident
-// under a compression CTA keeps the SM from giving its shared memory back to L1, and the
-// value-range pass that follows then ran with a few KB of it (512^3 call: 287 us against
-// 244 us); released by the value-range pass, the compression kernel gained nothing.
+// stream order. grid_release() lets the successor's CTAs start. The set-up, planning and
+// value-range kernels call it, after grid_wait(), which also orders the successor's early
+// loads after everything before the call. The two large kernels do not: a set-up CTA
+// resident under a compression CTA keeps the SM from giving its shared memory back to L1,
+// and the value-range pass that follows then ran with a few KB of it (512^3 call: 287 us
+// against 244 us).
 // Whole calls with plain launches and with these: 2^20 values compressed 22.3 -> 12.8 us,
 // decompressed 14.4 -> 9.7 us; 512^3 compressed 251.5 -> 244.5 us.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

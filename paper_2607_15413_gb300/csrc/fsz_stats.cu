@@ -180,7 +180,9 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
       chunk(in + e0, uint32_t(min(n - e0, uint64_t(kCChunkElems))));
     }
     deposit(0, 0, uint32_t(gn));
+    // (the set-up kernel has completed: the compression kernel may take its first tickets)
     grid_wait();
+    grid_release();
     __syncthreads();
     if (threadIdx.x == 0) publish(0);
   } else {

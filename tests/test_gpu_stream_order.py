@@ -84,3 +84,31 @@ def test_graph_of_chained_batches_replays(fszlib):
             ref, nb = fszlib.compress(x, 1e-3, fszlib.EB_REL)
             assert int(c.sizes[i]) == nb and torch.equal(c.arena[c.offsets[i]:c.offsets[i] + nb], ref)
             assert torch.equal(d.output(i), fszlib.decompress(ref, n=x.numel()))
+
+
+@pytest.mark.parametrize("n", [1, 8192 * 3 + 7, 8192 * 700 + 11])
+def test_a_refused_field_between_good_ones(fszlib, n):
+    """The compression kernel takes its first chunks before the field's step is known: a field
+    that then has none writes nothing, and the calls around it are whole."""
+    dev = _cuda()
+    good = torch.from_numpy(inputs.sinusoids(n, seed=2)).to(dev)
+    cap, dims = fszlib.fsz_compress_bound(n), fszlib.make_dims((n,))
+    want = fszlib.compress(good, 1e-3)[0].clone()
+    ws = fszlib.Workspace(n, dev)
+    sp = torch.cuda.current_stream().cuda_stream
+    x = good.clone()
+    outs = [torch.full((cap,), 0xA5, dtype=torch.uint8, device=dev) for _ in range(3)]
+    nb = torch.zeros(3, dtype=torch.int64, device=dev)
+    for k, out in enumerate(outs):
+        x.copy_(good)
+        if k == 1:
+            x[n - 1] = float("inf")
+        assert fszlib.fsz_compress(x.data_ptr(), dims, fszlib.EB_REL, 1e-3, out.data_ptr(), cap,
+                                   nb.data_ptr() + 8 * k, ws.ptr, ws.bytes, sp) == fszlib.OK
+        if k == 1:
+            assert fszlib.fsz_check(ws.ptr, sp) == fszlib.ERR_NONFINITE
+    assert fszlib.fsz_check(ws.ptr, sp) == fszlib.OK
+    assert nb.tolist() == [want.numel(), 0, want.numel()]
+    for out in (outs[0], outs[2]):
+        assert torch.equal(out[:want.numel()], want) and bool((out[want.numel():] == 0xA5).all())
+    assert bool((outs[1] == 0xA5).all())
