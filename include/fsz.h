@@ -250,7 +250,7 @@ fsz_status fsz_decompress_batched(const fsz_dfield* d_fields, uint32_t nfields,
 /* ------------------------------------------------------------------ graphs and schedules */
 
 /* A CUDA graph holding one batched call (no counterpart in the paper: it removes the
- * host launch cost of the call's memset and kernels). The graph records the pointers and
+ * host launch cost of the call's kernels). The graph records the pointers and
  * sizes given here; the field tables and buffers they point to are read when the graph
  * runs, so their contents may change between launches, but not their addresses or the
  * number of fields. The graph itself holds host-side and driver resources only. */

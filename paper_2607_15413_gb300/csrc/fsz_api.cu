@@ -351,7 +351,6 @@ fsz_status fsz_compress_batched(const fsz_cfield* d_fields, uint32_t nfields, ui
   const WsLayout L = ws_layout(n_total / kTile + nfields, nfields);
   if (ws_bytes < L.bytes) return FSZ_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(d_ws, 0, L.bytes, s) != cudaSuccess) return FSZ_ERR_CUDA;
   const KernelArgs a = make_args(d_ws, L);
   launch_plan_compress(a, d_fields, nfields, L.chunk_cap, s);
   const uint64_t max_chunks = n_total / kCChunkElems + nfields;
@@ -368,7 +367,6 @@ fsz_status fsz_decompress_batched(const fsz_dfield* d_fields, uint32_t nfields,
   const WsLayout L = ws_layout(n_total_capacity / kTile + nfields, nfields);
   if (ws_bytes < L.bytes) return FSZ_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(d_ws, 0, L.map_off, s) != cudaSuccess) return FSZ_ERR_CUDA;  // (control, fields)
   const KernelArgs a = make_args(d_ws, L);
   launch_plan_decompress(a, d_fields, nfields, L.chunk_cap, s);
   const uint64_t max_chunks = n_total_capacity / kDChunkElems + nfields;

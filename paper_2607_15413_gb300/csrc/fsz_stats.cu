@@ -191,6 +191,9 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
     // the grid, 142.4 us with ranges).
     grid_wait();
     const uint64_t total = a.ctrl->total_chunks;
+    for (uint64_t k = uint64_t(blockIdx.x) * kStatsThreads + threadIdx.x; k < kFlagStride * total;
+         k += uint64_t(gridDim.x) * kStatsThreads)
+      a.flags[k] = 0;  // (lookback flags, for the compression kernel)
     const uint64_t g0 = total * blockIdx.x / gridDim.x;
     const uint64_t gn = total * (blockIdx.x + 1) / gridDim.x - g0;
     for (uint64_t k0 = 0; k0 < gn; k0 += kSegChunks) {
@@ -520,35 +523,46 @@ inline int setup_grid(uint64_t nflags) {
 
 constexpr int kPlanThreads = 1024;
 
-// Batch planning (one CTA): per-field checks, an exclusive scan of the fields' chunk
-// counts (their ranges in the field-major ticket order) and the chunk -> field table.
+// Batch planning (one CTA): clears the control words and field records, per-field checks, an
+// exclusive scan of the fields' chunk counts (their ranges in the field-major ticket order)
+// and the chunk -> field table. Bound by latency (a chain of loads and barriers, 4 us for up
+// to 1024 fields).
 template <bool kCompress>
 __global__ void __launch_bounds__(kPlanThreads) fsz_plan_kernel(KernelArgs a, const void* d_fields,
                                                                 uint32_t nfields, uint64_t chunk_cap) {
   __shared__ uint64_t s_warp[kPlanThreads / 32];
+  __shared__ uint64_t s_first[kPlanThreads], s_count[kPlanThreads];
   __shared__ uint64_t s_carry;
+  __shared__ uint32_t s_status;  // the first error met
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) {
+    s_carry = 0;
+    s_status = 0;
+  }
+  __syncthreads();
   grid_wait();
   grid_release();
-  if (tid == 0) s_carry = 0;
-  __syncthreads();
+  uint32_t* const map = const_cast<uint32_t*>(a.chunk_field);
   for (uint32_t base = 0; base < nfields; base += kPlanThreads) {
     const uint32_t f = base + tid;
     uint64_t nch = 0;
     if (f < nfields) {
       FieldInfo* fi = a.fields + f;
+      FieldInfo rec = {};
       uint32_t st;
       if constexpr (kCompress) {
-        st = plan_cfield(fi, static_cast<const fsz_cfield*>(d_fields)[f]);
+        st = plan_cfield(&rec, static_cast<const fsz_cfield*>(d_fields)[f]);
       } else {
         const fsz_dfield d = static_cast<const fsz_dfield*>(d_fields)[f];
-        st = plan_dfield<false>(fi, static_cast<const uint8_t*>(d.in), d.in_bytes, d.out, d.out_capacity_elems);
+        st = plan_dfield<false>(&rec, static_cast<const uint8_t*>(d.in), d.in_bytes, d.out, d.out_capacity_elems);
       }
       if (st != FSZ_OK) {
-        set_error(a.ctrl, fi, st);
-        fi->nchunks = 0;
+        atomicCAS(&s_status, 0u, st);
+        rec.status = st;
+        rec.nchunks = 0;
       }
-      nch = fi->nchunks;
+      nch = rec.nchunks;
+      *fi = rec;
     }
     // block-wide exclusive scan of nch
     uint64_t inc = nch;
@@ -572,29 +586,29 @@ __global__ void __launch_bounds__(kPlanThreads) fsz_plan_kernel(KernelArgs a, co
     __syncthreads();
     const uint64_t first = s_carry + s_warp[warp] + inc - nch;
     if (f < nfields) a.fields[f].chunk_first = first;
+    s_first[tid] = first;
+    s_count[tid] = nch;
     __syncthreads();
     if (tid == kPlanThreads - 1) s_carry = first + nch;
+    // These fields' part of the chunk -> field table, one warp per field (their ranges are
+    // disjoint); nothing beyond the workspace's slots.
+    const uint32_t nb = min(nfields - base, uint32_t(kPlanThreads));
+    for (uint32_t k = uint32_t(warp); k < nb; k += uint32_t(kPlanThreads / 32)) {
+      const uint64_t c0 = s_first[k], c1 = min(c0 + s_count[k], chunk_cap);
+      for (uint64_t c = c0 + uint64_t(lane); c < c1; c += 32) map[c] = base + k;
+    }
     __syncthreads();
   }
   const uint64_t total = s_carry;
   if (tid == 0) {
-    a.ctrl->nfields = nfields;
-    if (total > chunk_cap) {
-      set_error(a.ctrl, nullptr, FSZ_ERR_WORKSPACE);
-      a.ctrl->total_chunks = 0;
-    } else {
-      a.ctrl->total_chunks = total;
-    }
+    Ctrl c = {};
+    c.status = total > chunk_cap && s_status == 0 ? uint32_t(FSZ_ERR_WORKSPACE) : s_status;
+    c.nfields = nfields;
+    c.total_chunks = total > chunk_cap ? 0 : total;
+    *a.ctrl = c;
   }
   if (total > chunk_cap) return;
-  // The chunk -> field table, one warp per field (the fields' ranges are disjoint), so
-  // that the fields' record loads overlap rather than follow one another.
-  uint32_t* map = const_cast<uint32_t*>(a.chunk_field);
-  for (uint32_t f = uint32_t(warp); f < nfields; f += uint32_t(kPlanThreads / 32)) {
-    const FieldInfo* fi = a.fields + f;
-    const uint64_t c0 = fi->chunk_first, nc = fi->nchunks;
-    for (uint64_t k = uint64_t(lane); k < nc; k += 32) map[c0 + k] = f;
-  }
+  __syncthreads();  // (the control words before an empty field's error)
   if constexpr (kCompress) {
     for (uint32_t f = tid; f < nfields; f += kPlanThreads) {
       FieldInfo* fi = a.fields + f;
