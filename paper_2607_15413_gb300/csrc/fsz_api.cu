@@ -115,18 +115,20 @@ fsz_status check_compress(const float* d_in, fsz_dims dims, fsz_eb_mode mode, do
   return FSZ_OK;
 }
 
-// Value-range pass and step for one field, with its switched-off features recorded in
+// Value-range pass and step (early: left to encode_one) for one field, with its switched-off features recorded in
 // the workspace's field record (read by the compression kernel and the preamble).
 fsz_status prepare_one(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double eb,
                        uint32_t features_off, void* d_out, uint64_t out_capacity,
-                       uint64_t* d_out_bytes, void* d_ws, uint64_t ws_bytes, fsz_stream stream) {
+                       uint64_t* d_out_bytes, void* d_ws, uint64_t ws_bytes, fsz_stream stream,
+                       bool early = false) {
   CompressCall call;
   fsz_status st = check_compress(d_in, dims, mode, eb, d_out, out_capacity, d_ws, ws_bytes, &call,
                                  features_off);
   if (st != FSZ_OK) return st;
   call.desc.out_bytes = d_out_bytes;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const KernelArgs a = make_args(d_ws, call.L);
+  KernelArgs a = make_args(d_ws, call.L);
+  a.early = early;
   launch_setup_compress(a, call.desc, call.L.chunk_cap, s);  // (clears the workspace it uses)
   if (call.desc.nchunks > 0) launch_stats(a, d_in, call.desc.n, s);
   return launched();
@@ -235,7 +237,7 @@ fsz_status fsz_compress_features(const float* d_in, fsz_dims dims, fsz_eb_mode m
                                  uint64_t* d_out_bytes, void* d_ws, uint64_t ws_bytes,
                                  fsz_stream stream) {
   fsz_status st = prepare_one(d_in, dims, mode, eb, features_off, d_out, out_capacity, d_out_bytes,
-                              d_ws, ws_bytes, stream);
+                              d_ws, ws_bytes, stream, true);
   if (st != FSZ_OK) return st;
   return encode_one(d_in, dims, mode, eb, features_off, d_out, out_capacity, d_ws, ws_bytes, stream, true);
 }

@@ -169,7 +169,9 @@ struct KernelArgs {
   uint64_t* flags;       // compression: lookback flags
   uint32_t* sums;        // decompression: payload bytes of each chunk,
   uint32_t* block_sums;  // ... and of each kSumBlock consecutive ones
-  bool early = false;   // compression of one field: start under the value-range pass
+  // compression of one field: the compression kernel starts under the value-range pass and
+  // derives the step itself
+  bool early = false;
   uint64_t skip_chunk;  // test hook: this chunk publishes no flag (decompression: no record)
   uint64_t timeout_ns;  // bound on every spin-wait
   // multipass compression only: the four variants' tile costs, variant-major (given_T
@@ -560,10 +562,76 @@ __device__ __forceinline__ float key_float(uint32_t k) {
   return __uint_as_float(u);
 }
 
+// ------------------------------------------------------------------ quantization step
+
+struct FieldStep {
+  double eb;
+  float e, s, r;
+  uint32_t Q;
+};
+
+// Derives eb, e, s = 2e and r = fl(1/s) from the field's range (reading of Sec. 5.1 and
+// of the error-bound argument of Sec. 4.2.2): ABS takes eb as given, REL takes
+// REL x (max - min) in float64 (REL x |max|, or REL, for a constant field). The half step
+// e = eb (1 - eps) rounded toward zero, eps = (3Q + 4) 2^-23, Q = ceil(A / (2 eb (1 -
+// c))) + 1, A = max |d|, with the cap c = 2^-4 where that gives eps <= 2^-4 and c = 2^-1
+// (eps <= 2^-1) otherwise: the two float32 roundings of quantization and reconstruction
+// then stay inside eb for every |q| <= Q.
+__device__ __forceinline__ uint32_t derive_step(const FieldInfo& f, FieldStep* p) {
+  if (f.max_abs_bits >= 0x7f800000u) return FSZ_ERR_NONFINITE;
+  float vmin = 0.0f, vmax = 0.0f;
+  if (f.n > 0) {
+    vmin = key_float(~f.min_inv_key);
+    vmax = key_float(f.max_key);
+  }
+  double eb = f.eb_req;
+  if (f.mode == FSZ_EB_REL) {
+    double range = __dadd_rn(double(vmax), -double(vmin));
+    if (range > 0.0) {
+      eb = __dmul_rn(f.eb_req, range);
+    } else {
+      double mag = fabs(double(vmax));
+      eb = mag > 0.0 ? __dmul_rn(f.eb_req, mag) : f.eb_req;
+    }
+  }
+  if (!(eb > 0.0) || isinf(eb)) return FSZ_ERR_EB_TOO_SMALL;
+  const double two100 = 1267650600228229401496703205376.0;  // 2^100
+  double eb_eff = eb < two100 ? eb : two100;
+  double A = fmax(fabs(double(vmin)), fabs(double(vmax)));
+  // first tier: K = A / (2 eb (1 - 2^-4)), eps <= 2^-4
+  double K = __ddiv_rn(A, __dmul_rn(__dmul_rn(2.0, eb_eff), 0.9375));
+  uint32_t Q = 0;
+  if (K <= double(kQmax1) && uint32_t(ceil(K)) + 1u <= kQmax1) {
+    Q = uint32_t(ceil(K)) + 1u;
+  } else {
+    // second tier, for fields the first refuses: K = A / (2 eb (1 - 2^-1)), eps <= 2^-1
+    K = __ddiv_rn(A, __dmul_rn(__dmul_rn(2.0, eb_eff), 0.5));
+    if (!(K <= double(kQmax2))) return FSZ_ERR_EB_TOO_SMALL;
+    Q = uint32_t(ceil(K)) + 1u;
+    if (Q > kQmax2) return FSZ_ERR_EB_TOO_SMALL;
+  }
+  double eps = __dmul_rn(double(3u * Q + 4u), 1.1920928955078125e-07);  // x 2^-23, exact
+  double x = __dmul_rn(eb_eff, __dadd_rn(1.0, -eps));
+  float e = __double2float_rz(x);
+  if (!(e >= 7.888609052210118e-31f)) return FSZ_ERR_EB_TOO_SMALL;  // 2^-100
+  float s = __fmul_rn(2.0f, e);
+  *p = FieldStep{eb, e, s, __fdiv_rn(1.0f, s), Q};
+  return FSZ_OK;
+}
+
+__device__ __forceinline__ void store_step(FieldInfo* fi, const FieldStep& p) {
+  fi->eb = p.eb;
+  fi->e = p.e;
+  fi->s = p.s;
+  fi->r = p.r;
+  fi->Q = p.Q;
+}
+
 // 64-byte preamble of this library's stream (little-endian; written once per field by the
 // CTA that finishes the field's last chunk), and the field's total size.
-// `tile_blocks`: rate bytes per tile.
-__device__ __forceinline__ void write_preamble(FieldInfo* fi, uint64_t data_bytes, int tile_blocks = 8) {
+// `step`: the field's s; `tile_blocks`: rate bytes per tile.
+__device__ __forceinline__ void write_preamble(FieldInfo* fi, uint64_t data_bytes, float step,
+                                               int tile_blocks = 8) {
   uint32_t w[16];
   w[0] = 0x315A5346u;  // "FSZ1"
   w[1] = 1u | (fi->ndim << 16) | (fi->mode << 24);
@@ -578,7 +646,7 @@ __device__ __forceinline__ void write_preamble(FieldInfo* fi, uint64_t data_byte
   const uint64_t eb = static_cast<uint64_t>(__double_as_longlong(fi->eb_req));
   w[10] = uint32_t(eb);
   w[11] = uint32_t(eb >> 32);
-  w[12] = __float_as_uint(fi->s);
+  w[12] = __float_as_uint(step);
   w[13] = fi->features_off;  // switched-off features and the tile configuration
   w[14] = uint32_t(data_bytes);
   w[15] = uint32_t(data_bytes >> 32);

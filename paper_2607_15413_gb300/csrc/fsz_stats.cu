@@ -13,63 +13,14 @@ namespace {
 
 constexpr int kStatsThreads = 256;
 
-// Derives eb, e, s = 2e and r = fl(1/s) from the field's range (reading of Sec. 5.1 and
-// of the error-bound argument of Sec. 4.2.2): ABS takes eb as given, REL takes
-// REL x (max - min) in float64 (REL x |max|, or REL, for a constant field). The half step
-// e = eb (1 - eps) rounded toward zero, eps = (3Q + 4) 2^-23, Q = ceil(A / (2 eb (1 -
-// c))) + 1, A = max |d|, with the cap c = 2^-4 where that gives eps <= 2^-4 and c = 2^-1
-// (eps <= 2^-1) otherwise: the two float32 roundings of quantization and reconstruction
-// then stay inside eb for every |q| <= Q.
-__device__ uint32_t derive_params(FieldInfo* fi) {
-  if (fi->max_abs_bits >= 0x7f800000u) return FSZ_ERR_NONFINITE;
-  float vmin = 0.0f, vmax = 0.0f;
-  if (fi->n > 0) {
-    vmin = key_float(~fi->min_inv_key);
-    vmax = key_float(fi->max_key);
-  }
-  double eb = fi->eb_req;
-  if (fi->mode == FSZ_EB_REL) {
-    double range = __dadd_rn(double(vmax), -double(vmin));
-    if (range > 0.0) {
-      eb = __dmul_rn(fi->eb_req, range);
-    } else {
-      double mag = fabs(double(vmax));
-      eb = mag > 0.0 ? __dmul_rn(fi->eb_req, mag) : fi->eb_req;
-    }
-  }
-  if (!(eb > 0.0) || isinf(eb)) return FSZ_ERR_EB_TOO_SMALL;
-  const double two100 = 1267650600228229401496703205376.0;  // 2^100
-  double eb_eff = eb < two100 ? eb : two100;
-  double A = fmax(fabs(double(vmin)), fabs(double(vmax)));
-  // first tier: K = A / (2 eb (1 - 2^-4)), eps <= 2^-4
-  double K = __ddiv_rn(A, __dmul_rn(__dmul_rn(2.0, eb_eff), 0.9375));
-  uint32_t Q = 0;
-  if (K <= double(kQmax1) && uint32_t(ceil(K)) + 1u <= kQmax1) {
-    Q = uint32_t(ceil(K)) + 1u;
-  } else {
-    // second tier, for fields the first refuses: K = A / (2 eb (1 - 2^-1)), eps <= 2^-1
-    K = __ddiv_rn(A, __dmul_rn(__dmul_rn(2.0, eb_eff), 0.5));
-    if (!(K <= double(kQmax2))) return FSZ_ERR_EB_TOO_SMALL;
-    Q = uint32_t(ceil(K)) + 1u;
-    if (Q > kQmax2) return FSZ_ERR_EB_TOO_SMALL;
-  }
-  double eps = __dmul_rn(double(3u * Q + 4u), 1.1920928955078125e-07);  // x 2^-23, exact
-  double x = __dmul_rn(eb_eff, __dadd_rn(1.0, -eps));
-  float e = __double2float_rz(x);
-  if (!(e >= 7.888609052210118e-31f)) return FSZ_ERR_EB_TOO_SMALL;  // 2^-100
-  float s = __fmul_rn(2.0f, e);
-  fi->eb = eb;
-  fi->e = e;
-  fi->s = s;
-  fi->r = __fdiv_rn(1.0f, s);
-  fi->Q = Q;
-  return FSZ_OK;
-}
-
 __device__ __forceinline__ void finish_field(Ctrl* ctrl, FieldInfo* fi) {
   if (fi->status != 0) return;
-  uint32_t st = derive_params(fi);
-  if (st != FSZ_OK) set_error(ctrl, fi, st);
+  FieldStep p;
+  const uint32_t st = derive_step(*fi, &p);
+  if (st != FSZ_OK)
+    set_error(ctrl, fi, st);
+  else
+    store_step(fi, p);
 }
 
 // A CTA's chunks are taken in segments of up to kSegChunks. For a batch, the segment's chunk
@@ -159,6 +110,7 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
       atomicMax(&fi->max_key, float_key(h));
     }
     atomicMax(&fi->max_abs_bits, m);
+    if (kSingle && a.early) return;  // (the compression kernel behind this one derives the step)
     __threadfence();
     const uint32_t prev = atomicAdd(&fi->done_chunks, s_cnt[k]);
     if (uint64_t(prev) + s_cnt[k] == fi->nchunks) {
@@ -333,7 +285,7 @@ __device__ uint32_t plan_dfield(FieldInfo* fi, const uint8_t* in, uint64_t in_by
 // A valid field of zero elements: its step, its 64-byte stream and its size.
 __device__ void finish_empty_field(Ctrl* ctrl, FieldInfo* fi) {
   finish_field(ctrl, fi);
-  if (fi->status == 0) write_preamble(fi, 0);
+  if (fi->status == 0) write_preamble(fi, 0, fi->s);
 }
 
 // One-field set-up for compression: the descriptor is validated on the host, so this
