@@ -112,3 +112,47 @@ def test_a_refused_field_between_good_ones(fszlib, n):
     for out in (outs[0], outs[2]):
         assert torch.equal(out[:want.numel()], want) and bool((out[want.numel():] == 0xA5).all())
     assert bool((outs[1] == 0xA5).all())
+
+
+@pytest.mark.parametrize("n", [300, 8192 * 40 + 3])
+def test_captured_behind_copies_and_joins(fszlib, n):
+    """A captured call whose first kernel follows a copy, a fill, or the join of two streams."""
+    dev = _cuda()
+    host = [torch.from_numpy(inputs.sinusoids(n, seed=s)).pin_memory() for s in (3, 4)]
+    cap, dims = fszlib.fsz_compress_bound(n), fszlib.make_dims((n,))
+    x, y = torch.zeros(n, device=dev), torch.zeros(n, device=dev)
+    back = torch.zeros(max(n, 4), device=dev)
+    a, b = (torch.zeros(cap, dtype=torch.uint8, device=dev) for _ in range(2))
+    nb = torch.zeros(2, dtype=torch.int64, device=dev)
+    wa, wb = fszlib.Workspace(n, dev), fszlib.Workspace(n, dev)
+    feed = host[0].clone().pin_memory()
+    fszlib.compress(host[0].to(dev), 1e-3)              # (launch settings, before the capture)
+    fszlib.decompress(fszlib.compress(host[0].to(dev), 1e-3)[0], n=n)
+
+    def comp(src, out, k, ws):
+        sp = torch.cuda.current_stream().cuda_stream
+        return fszlib.fsz_compress(src.data_ptr(), dims, fszlib.EB_REL, 1e-3, out.data_ptr(), cap,
+                                   nb.data_ptr() + 8 * k, ws.ptr, ws.bytes, sp)
+
+    g = torch.cuda.CUDAGraph()
+    main, side = torch.cuda.Stream(dev), torch.cuda.Stream(dev)
+    with torch.cuda.graph(g, stream=main):
+        x.copy_(feed, non_blocking=True)
+        assert comp(x, a, 0, wa) == fszlib.OK           # behind a copy
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            y.copy_(x)
+            y.mul_(3.0)
+        back.zero_()
+        main.wait_stream(side)
+        assert comp(y, b, 1, wb) == fszlib.OK           # behind a fill and another stream
+        assert fszlib.fsz_decompress(b.data_ptr(), cap, back.data_ptr(), back.numel(), wa.ptr, wa.bytes,
+                                     main.cuda_stream) == fszlib.OK
+    for h in host:
+        feed.copy_(h)
+        g.replay()
+        torch.cuda.synchronize()
+        for src, out, k in ((h.to(dev), a, 0), (h.to(dev) * 3.0, b, 1)):
+            ref, m = fszlib.compress(src, 1e-3)
+            assert int(nb[k]) == m and torch.equal(out[:m], ref[:m])
+        assert torch.equal(back[:n], fszlib.decompress(b[:int(nb[1])].clone(), n=n))
