@@ -115,8 +115,9 @@ fsz_status check_compress(const float* d_in, fsz_dims dims, fsz_eb_mode mode, do
   return FSZ_OK;
 }
 
-// Value-range pass and step (early: left to encode_one) for one field, with its switched-off features recorded in
-// the workspace's field record (read by the compression kernel and the preamble).
+// Value-range pass and step (early: the step is left to encode_one) for one field, with its
+// switched-off features recorded in the workspace's field record (read by the compression
+// kernel and the preamble).
 fsz_status prepare_one(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double eb,
                        uint32_t features_off, void* d_out, uint64_t out_capacity,
                        uint64_t* d_out_bytes, void* d_ws, uint64_t ws_bytes, fsz_stream stream,

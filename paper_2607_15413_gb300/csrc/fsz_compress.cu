@@ -671,7 +671,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
                   }
                 }
               }
-              if (lane == 0 && (ci.flags & kInfoLast)) write_preamble(ci.fi, excl + tot, a.early ? step_s : ci.fi->s, Cfg::kT);
+              if (lane == 0 && (ci.flags & kInfoLast))
+                write_preamble(ci.fi, excl + tot, a.early ? step_s : ci.fi->s, Cfg::kT);
             }
           }
           // the runs are read: their ring space goes back to the compute warps

@@ -1,11 +1,12 @@
 // Internal definitions shared by the FSZ CUDA kernels (sm_103a).
 //
-// Work decomposition (GB300 design, not the paper's): a persistent CTA takes chunks of
-// tiles by an atomic ticket, stages them in shared memory with 1-D TMA bulk copies
-// (mbarrier-tracked) and gives each warp one 256-element tile at a time. Lane j of the
-// warp owns the 8 consecutive elements 8j..8j+7, so the 4 lanes 4g..4g+3 hold block g
-// (Sec. 3.1: a tile is 8 blocks of 32 elements). Residual chains stay in registers; a
-// shuffle carries the state across lane and block boundaries.
+// Work decomposition (GB300 design, not the paper's): a persistent CTA takes chunks of 8192
+// elements by an atomic ticket, stages them in shared memory (compression: cp.async of the
+// values; decompression: 1-D TMA bulk copies of the payload) and gives each warp a quad of
+// 1024 elements at a time: four tiles of the default configuration (Sec. 3.1: a tile is 8
+// blocks of 32 elements). Lane L of the warp owns elements 32 L .. 32 L + 31: one block, so a
+// block's bits are transposed without exchanging anything between lanes. Residual chains stay
+// in registers; a shuffle carries the state across block boundaries.
 #pragma once
 
 #include <cstdint>
@@ -756,7 +757,12 @@ void launch_cost_pass(const KernelArgs& a, int variant, uint32_t* costs, cudaStr
 // Decoder instances: the full method's; one that also decodes streams without the
 // cross-block state; one for a pre-zeroed output that skips all-zero tiles; one for streams of
 // any tile configuration.
-enum DecompressKind { kDecompressFull = 0, kDecompressAny = 1, kDecompressPrezeroed = 2, kDecompressTiled = 3 };
+enum DecompressKind {
+  kDecompressFull = 0,
+  kDecompressAny = 1,
+  kDecompressPrezeroed = 2,
+  kDecompressTiled = 3
+};
 void launch_decompress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st,
                        DecompressKind kind = kDecompressFull);
 // Single-field set-up: fills in the control words and the field record; for compression it

@@ -2,7 +2,8 @@
 //
 // fsz_stats_kernel: min, max and finiteness of every field (Sec. 5.1: eb = REL x (max -
 // min)), then the float32-safe quantization step of each field, derived on the device
-// by whichever CTA finishes the field's last chunk, so the host never waits.
+// (by whichever CTA finishes the field's last chunk or, in a one-field call, by the compression
+// kernel), so the host never waits.
 // Set-up kernels (one field) and planning kernels (a batch) fill the per-field state and
 // the chunk -> field table that every later kernel of the call reads.
 #include "fsz_internal.cuh"
@@ -288,11 +289,9 @@ __device__ void finish_empty_field(Ctrl* ctrl, FieldInfo* fi) {
   if (fi->status == 0) write_preamble(fi, 0, fi->s);
 }
 
-// One-field set-up for compression: the descriptor is validated on the host, so this
-// copies it into the workspace.
-// Set-up of a single-field compression: thread 0 of CTA 0 clears the control words and the field
-// record and fills them in; every other thread clears the lookback flags (nflags words),
-// so that the call needs no separate memset.
+// Set-up of a single-field compression, whose descriptor the host has validated: thread 0 of
+// CTA 0 clears the control words and the field record and fills them in; every other thread
+// clears the lookback flags (nflags words), so that the call needs no separate memset.
 constexpr int kSetupThreads = 256;
 static_assert(sizeof(Ctrl) <= 256 && sizeof(Ctrl) % 8 == 0 && sizeof(FieldInfo) % 8 == 0,
               "control words and field record clear as 8-byte words");
@@ -396,7 +395,8 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(Kern
   uint64_t h[kChunksPerWarp];
   if constexpr (!kTiled) {
 #pragma unroll
-    for (int k = 0; k < kChunksPerWarp; ++k) h[k] = load_unit(unit(blockIdx.x, k), room);  // (issued with n's load)
+    for (int k = 0; k < kChunksPerWarp; ++k)  // (issued with n's load)
+      h[k] = load_unit(unit(blockIdx.x, k), room);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     FieldInfo f = {};
@@ -506,7 +506,8 @@ __global__ void __launch_bounds__(kPlanThreads) fsz_plan_kernel(KernelArgs a, co
         st = plan_cfield(&rec, static_cast<const fsz_cfield*>(d_fields)[f]);
       } else {
         const fsz_dfield d = static_cast<const fsz_dfield*>(d_fields)[f];
-        st = plan_dfield<false>(&rec, static_cast<const uint8_t*>(d.in), d.in_bytes, d.out, d.out_capacity_elems);
+        st = plan_dfield<false>(&rec, static_cast<const uint8_t*>(d.in), d.in_bytes, d.out,
+                                d.out_capacity_elems);
       }
       if (st != FSZ_OK) {
         atomicCAS(&s_status, 0u, st);
