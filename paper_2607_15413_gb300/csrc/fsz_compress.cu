@@ -465,6 +465,51 @@ __device__ __forceinline__ void encode_block(const QuadPlan& P, uint32_t blk) {
   }
 }
 
+// Copies the runs of compute warps W0 .. W0 + N - 1 of the chunk in slot b to the stream, base
+// being the chunk's place there. The runs' parameters are read side by side (one lane each), then
+// the words of all of them, 4 per lane and run at a time: run after run, each waited for its own
+// parameters and first words, and a launch of few chunks for that on its way out (2^20 values
+// 12.7 -> 12.2 us, 31 MB field 23.3 -> 22.9 us, 512^3 equal; 2 or 8 words: the same, 0.8 % slower
+// at 512^3).
+template <int W0, int N>
+__device__ __forceinline__ void place_runs(CompressSmem& S, int b, uint8_t* base, int lane) {
+  if constexpr (N > 0) {
+    constexpr int kPer = 4;
+    uint32_t nw = 0, src = 0, off = 0;
+    if (lane < N) {
+      nw = S.qlen[b][W0 + lane] >> 2;
+      src = smem_u32(S.ring[W0 + lane]) + S.qring[b][W0 + lane].x;
+      off = S.qoff[b][W0 + lane];
+    }
+    const uint32_t most = __reduce_max_sync(FULL, nw);
+    uint32_t n[N], s[N], o[N];
+#pragma unroll
+    for (int w = 0; w < N; ++w) {
+      n[w] = __shfl_sync(FULL, nw, w);
+      s[w] = __shfl_sync(FULL, src, w) + 4 * lane;
+      o[w] = __shfl_sync(FULL, off, w) + 4 * lane;
+    }
+    for (uint32_t q0 = uint32_t(lane); q0 < most + uint32_t(lane); q0 += 32 * kPer) {
+      uint32_t v[N][kPer];
+#pragma unroll
+      for (int w = 0; w < N; ++w) {
+#pragma unroll
+        for (int k = 0; k < kPer; ++k)
+          if (q0 + 32 * k < n[w]) v[w][k] = lds32(s[w] + 128 * k);
+        s[w] += 128 * kPer;
+      }
+#pragma unroll
+      for (int w = 0; w < N; ++w) {
+        uint32_t* dst = reinterpret_cast<uint32_t*>(base + o[w]);
+#pragma unroll
+        for (int k = 0; k < kPer; ++k)
+          if (q0 + 32 * k < n[w]) dst[32 * k] = v[w][k];
+        o[w] += 128 * kPer;
+      }
+    }
+  }
+}
+
 // kGiven: the multipass evaluation's encoding pass (selection from a.given_costs).
 // kFeat: fields' switched-off features honoured; without it the full method is compiled
 // with none of that handling. Cfg: the tile configuration. (Every configuration through this
@@ -653,24 +698,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
               if (lane == 0) set_error(a.ctrl, ci.fi, FSZ_ERR_CAPACITY);
             } else {
               uint8_t* const base = ci.out + ci.data_base + excl;
-              for (int w = kResolverRuns; w < kWarps; ++w) {
-                const uint32_t nw = S.qlen[b][w] >> 2;
-                const uint32_t src = smem_u32(S.ring[w]) + S.qring[b][w].x;
-                uint32_t* dst = reinterpret_cast<uint32_t*>(base + S.qoff[b][w]);
-                for (uint32_t q0 = 0; q0 < nw; q0 += 128) {  // 4 words per lane in flight
-                  uint32_t v[4];
-#pragma unroll
-                  for (int k = 0; k < 4; ++k) {
-                    const uint32_t q = q0 + 32 * k + lane;
-                    if (q < nw) v[k] = lds32(src + 4 * q);
-                  }
-#pragma unroll
-                  for (int k = 0; k < 4; ++k) {
-                    const uint32_t q = q0 + 32 * k + lane;
-                    if (q < nw) dst[q] = v[k];
-                  }
-                }
-              }
+              place_runs<kResolverRuns, kWarps - kResolverRuns>(S, b, base, lane);
               if (lane == 0 && (ci.flags & kInfoLast))
                 write_preamble(ci.fi, excl + tot, a.early ? step_s : ci.fi->s, Cfg::kT);
             }
@@ -747,24 +775,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
         const uint32_t tot = S.set_tot[b];
         if ((flags & (kInfoOk | kInfoSkip)) == kInfoOk && ci.data_base + excl + tot <= ci.cap) {
           uint8_t* const base = ci.out + ci.data_base + excl;
-          for (int w = 0; w < kResolverRuns; ++w) {
-            const uint32_t nw = S.qlen[b][w] >> 2;
-            const uint32_t src = smem_u32(S.ring[w]) + S.qring[b][w].x;
-            uint32_t* dst = reinterpret_cast<uint32_t*>(base + S.qoff[b][w]);
-            for (uint32_t q0 = 0; q0 < nw; q0 += 128) {
-              uint32_t v[4];
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const uint32_t q = q0 + 32 * k + lane;
-                if (q < nw) v[k] = lds32(src + 4 * q);
-              }
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const uint32_t q = q0 + 32 * k + lane;
-                if (q < nw) dst[q] = v[k];
-              }
-            }
-          }
+          place_runs<0, kResolverRuns>(S, b, base, lane);
         }
         __syncwarp();
         if (lane < kResolverRuns) {
