@@ -373,7 +373,7 @@ fsz_status fsz_decompress_batched(const fsz_dfield* d_fields, uint32_t nfields,
   const KernelArgs a = make_args(d_ws, L);
   launch_plan_decompress(a, d_fields, nfields, L.chunk_cap, s);
   const uint64_t max_chunks = n_total_capacity / kDChunkElems + nfields;
-  launch_sizes(a, max_chunks, s);
+  launch_sizes(a, d_fields, nfields, L.chunk_cap, max_chunks, s);
   launch_decompress(a, max_chunks, s);
   return launched();
 }

@@ -767,12 +767,13 @@ void launch_decompress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st
                        DecompressKind kind = kDecompressFull);
 // Single-field set-up: fills in the control words and the field record; for compression it
 // clears the lookback flags, for decompression it sizes the chunks' payloads (no memset of
-// the workspace needed). launch_sizes: the sizing of a planned batch.
+// the workspace needed). launch_sizes: the sizing of a batch behind its planning kernel.
 void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t chunk_cap, cudaStream_t st);
 // tiled: any tile configuration's stream (of at most max_chunks chunks).
 void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st,
                              bool tiled = false);
-void launch_sizes(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st);
+void launch_sizes(const KernelArgs& a, const fsz_dfield* d_fields, uint32_t nfields, uint64_t chunk_cap,
+                  uint64_t max_chunks, cudaStream_t st);
 void launch_plan_compress(const KernelArgs& a, const fsz_cfield* d_fields, uint32_t nfields,
                           uint64_t chunk_cap, cudaStream_t st);
 void launch_plan_decompress(const KernelArgs& a, const fsz_dfield* d_fields, uint32_t nfields,

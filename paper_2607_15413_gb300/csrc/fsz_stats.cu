@@ -427,13 +427,77 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(Kern
   }
 }
 
-// A planned batch.
-__global__ void __launch_bounds__(kSizeThreads) fsz_sizes_kernel(KernelArgs a) {
+// The chunk ranges of a batch of up to kSizeThreads fields, worked out from the descriptors by a
+// CTA for itself.
+struct SelfPlan {
+  uint64_t warp_sum[kSizeWarps];
+  uint64_t total;
+  uint64_t first[kSizeThreads];      // a field's first chunk,
+  uint64_t tiles[kSizeThreads];      // ... its tiles,
+  const uint8_t* stream[kSizeThreads];
+};
+
+// Fills S by the rules of the planning kernel; returns the chunks (none if they exceed the
+// workspace's slots, as it does).
+__device__ uint64_t self_plan(SelfPlan& S, const fsz_dfield* d_fields, uint32_t nfields, uint64_t chunk_cap) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint64_t nch = 0;
+  if (tid < nfields) {
+    const fsz_dfield d = d_fields[tid];
+    FieldInfo rec = {};
+    const uint32_t st = plan_dfield<false>(&rec, static_cast<const uint8_t*>(d.in), d.in_bytes, d.out,
+                                           d.out_capacity_elems);
+    nch = st == FSZ_OK ? rec.nchunks : 0;
+    S.tiles[tid] = rec.T;
+    S.stream[tid] = rec.sin;
+  }
+  uint64_t inc = nch;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= uint32_t(o)) inc += y;
+  }
+  if (lane == 31) S.warp_sum[warp] = inc;
+  __syncthreads();
+  uint64_t first = inc - nch;
+  for (uint32_t w = 0; w < warp; ++w) first += S.warp_sum[w];
+  S.first[tid] = first;
+  if (tid == kSizeThreads - 1) S.total = first + nch;
+  __syncthreads();
+  return S.total > chunk_cap ? 0 : S.total;
+}
+
+// The field of chunk c (below the total): the last one that begins at or before it.
+__device__ __forceinline__ uint32_t field_of_chunk(const SelfPlan& S, uint32_t nfields, uint64_t c) {
+  uint32_t f = 0;
+#pragma unroll
+  for (uint32_t s = kSizeThreads / 2; s > 0; s >>= 1)
+    if (f + s < nfields && S.first[f + s] <= c) f += s;
+  return f;
+}
+
+// A batch. Its planning kernel is 4 to 5 us of loads that wait for one another in one CTA: with
+// up to kSizeThreads fields, a thread each, the sizing CTAs plan for themselves under it instead
+// of waiting for its records and its chunk -> field table, unless they are so many that reading
+// every field in each costs more (whole calls behind it and for themselves: 32 fields of 258 MB
+// 62.8 / 60.5 us; 512 of 256 KB, 128 CTAs: 47.4 / 44.5; 128 of 4 MB, 608 CTAs: 105.6 / 104.6;
+// 256 of 4 MB: 193.4 / 196.3). The value-range pass of a compression does not do it: with the
+// registers and the shared memory that takes, the 32 fields went from 118.7 to 121.0 us.
+constexpr uint32_t kSelfPlanReads = 128 * 608;  // fields x CTAs
+__global__ void __launch_bounds__(kSizeThreads) fsz_sizes_kernel(KernelArgs a, const fsz_dfield* d_fields,
+                                                                 uint32_t nfields, uint64_t chunk_cap) {
   __shared__ uint32_t s_sum[kSumBlock];
+  __shared__ SelfPlan plan;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  grid_wait();
+  const bool own = nfields <= uint32_t(kSizeThreads) && nfields * gridDim.x <= kSelfPlanReads;
+  uint64_t total;
+  if (own) {
+    total = self_plan(plan, d_fields, nfields, chunk_cap);
+  } else {
+    grid_wait();
+    total = a.ctrl->total_chunks;
+  }
   grid_release();
-  const uint64_t total = a.ctrl->total_chunks;
   for (uint64_t b = blockIdx.x; b * kSumBlock < total; b += gridDim.x) {
     uint32_t bytes[kChunksPerWarp];
 #pragma unroll
@@ -441,15 +505,18 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_sizes_kernel(KernelArgs a) {
       const uint64_t c = b * kSumBlock + kSizeWarps * k + warp;
       bytes[k] = 0;
       if (c < total) {
-        const FieldInfo* fi = a.fields + a.chunk_field[c];
-        const uint64_t t = (c - fi->chunk_first) * kDChunkTiles + lane;
-        if (t < fi->T)
-          bytes[k] = unit_bytes(__ldg(reinterpret_cast<const unsigned long long*>(fi->sin + 64) + t),
-                                32, 8, t);
+        const uint32_t f = own ? field_of_chunk(plan, nfields, c) : a.chunk_field[c];
+        const FieldInfo* fi = a.fields + f;
+        const uint8_t* in = own ? plan.stream[f] : fi->sin;
+        const uint64_t first = own ? plan.first[f] : fi->chunk_first, T = own ? plan.tiles[f] : fi->T;
+        const uint64_t t = (c - first) * kDChunkTiles + lane;
+        if (t < T)
+          bytes[k] = unit_bytes(__ldg(reinterpret_cast<const unsigned long long*>(in + 64) + t), 32, 8, t);
       }
     }
     write_chunk_sizes(a, b, total, bytes, s_sum);
   }
+  grid_wait();  // (this kernel completes after the planning kernel)
 }
 
 // CTAs of a sizing launch: one per kSumBlock chunks, at most four per SM.
@@ -610,8 +677,10 @@ void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream
                    chunk_cap);
 }
 
-void launch_sizes(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st) {
-  launch_dependent(fsz_sizes_kernel, sizes_grid(max_chunks), kSizeThreads, 0, st, a);
+void launch_sizes(const KernelArgs& a, const fsz_dfield* d_fields, uint32_t nfields, uint64_t chunk_cap,
+                  uint64_t max_chunks, cudaStream_t st) {
+  launch_dependent(fsz_sizes_kernel, sizes_grid(max_chunks), kSizeThreads, 0, st, a, d_fields, nfields,
+                   chunk_cap);
 }
 
 void launch_plan_compress(const KernelArgs& a, const fsz_cfield* d_fields, uint32_t nfields,
