@@ -357,7 +357,7 @@ fsz_status fsz_compress_batched(const fsz_cfield* d_fields, uint32_t nfields, ui
   const KernelArgs a = make_args(d_ws, L);
   launch_plan_compress(a, d_fields, nfields, L.chunk_cap, s);
   const uint64_t max_chunks = n_total / kCChunkElems + nfields;
-  launch_stats_batch(a, max_chunks, s);
+  launch_stats_batch(a, d_fields, nfields, L.chunk_cap, max_chunks, s);
   launch_compress(a, max_chunks, s, kCompressFeatures);  // fields may switch features off
   return launched();
 }

@@ -739,9 +739,10 @@ LaunchCfg stats_cfg();
 LaunchCfg compress_cfg();
 LaunchCfg decompress_cfg();
 
-// One field (in, n), or the batch that the workspace describes.
+// One field (in, n), or a batch behind its planning kernel.
 void launch_stats(const KernelArgs& a, const float* in, uint64_t n, cudaStream_t st);
-void launch_stats_batch(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st);
+void launch_stats_batch(const KernelArgs& a, const fsz_cfield* d_fields, uint32_t nfields,
+                        uint64_t chunk_cap, uint64_t max_chunks, cudaStream_t st);
 // Compression kernel instances (feature-toggle builds of one kernel): the full method;
 // with switched-off features honoured per field (fsz_compress_features, batches); the
 // multipass evaluation's encoding pass (selection from a.given_costs).

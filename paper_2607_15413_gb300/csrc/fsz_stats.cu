@@ -24,6 +24,95 @@ __device__ __forceinline__ void finish_field(Ctrl* ctrl, FieldInfo* fi) {
     store_step(fi, p);
 }
 
+// n *= dk; false if the product exceeds kMaxElems (n itself does not). Without a 64-bit
+// division, which the single thread that plans a field would wait for.
+__device__ __forceinline__ bool times_dim(uint64_t* n, uint64_t dk) {
+  if (__umul64hi(*n, dk) != 0) return false;
+  *n *= dk;
+  return *n <= kMaxElems;
+}
+
+// Validates one compression descriptor and fills the field's shape (host-visible errors
+// of the one-field entry point are checked again here for batches).
+__device__ uint32_t plan_cfield(FieldInfo* fi, const fsz_cfield& d) {
+  fi->in = d.in;
+  fi->out = static_cast<uint8_t*>(d.out);
+  fi->cap = d.out_capacity;
+  fi->out_bytes = d.out_bytes;
+  fi->mode = d.mode;
+  fi->eb_req = d.eb;
+  fi->ndim = d.dims.ndim;
+  fi->nchunks = 0;
+  fi->features_off = d.features_off;
+  if (d.dims.ndim < 1 || d.dims.ndim > 3 || d.dims.reserved != 0 || !features_valid(d.features_off) ||
+      d.mode > 1 || !(d.eb > 0.0) || isinf(d.eb) || d.out == nullptr)
+    return FSZ_ERR_INVALID_ARG;
+  uint64_t n = 1;
+#pragma unroll
+  for (uint32_t k = 0; k < 3; ++k) {
+    if (k >= d.dims.ndim) continue;
+    const uint64_t dk = d.dims.dims[k];
+    if (!times_dim(&n, dk)) return FSZ_ERR_INVALID_ARG;
+    fi->dims[k] = dk;
+  }
+  if (n > kMaxElems) return FSZ_ERR_INVALID_ARG;
+  if ((reinterpret_cast<uintptr_t>(d.in) & 15) || (reinterpret_cast<uintptr_t>(d.out) & 15))
+    return FSZ_ERR_ALIGN;
+  if (n > 0 && d.in == nullptr) return FSZ_ERR_INVALID_ARG;
+  const uint64_t T = (n + kTile - 1) / kTile;
+  fi->n = n;
+  fi->T = T;
+  if (d.out_capacity < 64 + 8 * T) return FSZ_ERR_CAPACITY;
+  fi->nchunks = (T + kCChunkTiles - 1) / kCChunkTiles;
+  return FSZ_OK;
+}
+
+// The chunk ranges of a batch of up to kStatsPlanned fields, worked out from the descriptors by
+// each CTA of the value-range kernel for itself: its loads then run under the planning kernel (4 to
+// 5 us of loads that wait for one another in one CTA), which only the publication of the ranges
+// waits for. An instance of its own and no more fields, because 760 CTAs of 48 registers stream
+// at the copy peak only while the L1 has room for what they have in flight. Whole calls, behind
+// the planning kernel and for themselves: 8 fields of 256 KB 14.6 / 13.3 us, 32 of 512 KB
+// 20.2 / 18.3, 32 of 8 MB 108.9 / 107.4, 64 of 8 MB 211.3 / 207.7, 32 mixed ones of 258 MB in
+// all 118.9 / 118.9; with up to 256 fields, in one instance with the other way: 121.0.
+constexpr uint32_t kStatsPlanned = 64;
+struct StatsPlan {
+  uint64_t total;
+  uint64_t first[kStatsPlanned];      // a field's first chunk,
+  uint64_t n[kStatsPlanned];          // ... its elements,
+  const float* in[kStatsPlanned];
+};
+
+// Fills S by the rules of the planning kernel; returns the chunks (none if they exceed the
+// workspace's slots, as it does).
+__device__ uint64_t stats_plan(StatsPlan& S, const fsz_cfield* d_fields, uint32_t nfields,
+                               uint64_t chunk_cap) {
+  const uint32_t tid = threadIdx.x;
+  uint64_t nch = 0;
+  if (tid < nfields) {
+    FieldInfo rec = {};
+    if (plan_cfield(&rec, d_fields[tid]) == FSZ_OK) nch = rec.nchunks;
+    S.n[tid] = rec.n;
+    S.in[tid] = rec.in;
+  }
+  if (tid < kStatsPlanned) {
+    uint64_t inc = nch;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if ((tid & 31) >= uint32_t(o)) inc += y;
+    }
+    S.first[tid] = inc - nch;
+    if (tid == 31) S.total = inc;  // (of the first 32)
+  }
+  __syncthreads();
+  if (tid >= 32 && tid < kStatsPlanned) S.first[tid] += S.total;
+  __syncthreads();
+  if (tid == kStatsPlanned - 1) S.total = S.first[tid] + nch;
+  __syncthreads();
+  return S.total > chunk_cap ? 0 : S.total;
+}
+
 // A CTA's chunks are taken in segments of up to kSegChunks. For a batch, the segment's chunk
 // descriptors are read together at its start (two dependent loads for all of them instead
 // of two per chunk), and each field's partial range is left in shared memory; at the
@@ -40,9 +129,15 @@ struct StatsItem {
   uint32_t f;
 };
 
-template <bool kSingle>
-__global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs a, const float* in,
-                                                                       uint64_t n) {
+// kStatsSingle: the field src of n elements. kStatsBatch: the batch that the planning kernel has
+// recorded. kStatsBatchOwn: the batch of the nfields descriptors at src, n chunk slots in the
+// workspace.
+enum StatsKind { kStatsSingle = 0, kStatsBatch = 1, kStatsBatchOwn = 2 };
+
+template <int kKind>
+__global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs a, const void* src,
+                                                                       uint64_t n, uint32_t nfields) {
+  constexpr bool kSingle = kKind == kStatsSingle, kOwn = kKind == kStatsBatchOwn;
   constexpr int kStatsWarps = kStatsThreads / 32;
   __shared__ StatsItem s_item[kSegChunks];
   __shared__ float s_lo[kSegChunks][kStatsWarps], s_hi[kSegChunks][kStatsWarps];
@@ -130,7 +225,7 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
     const uint64_t gn = (total - blockIdx.x + gridDim.x - 1) / gridDim.x;
     for (uint64_t k = 0; k < gn; ++k) {
       const uint64_t e0 = (total - 1 - (blockIdx.x + k * gridDim.x)) * uint64_t(kCChunkElems);
-      chunk(in + e0, uint32_t(min(n - e0, uint64_t(kCChunkElems))));
+      chunk(static_cast<const float*>(src) + e0, uint32_t(min(n - e0, uint64_t(kCChunkElems))));
     }
     deposit(0, 0, uint32_t(gn));
     // (the set-up kernel has completed: the compression kernel may take its first tickets)
@@ -142,8 +237,14 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
     // A batch: each CTA takes one contiguous range of its chunks and so meets few fields
     // (a batch of 32 mixed fields of 258 MB in all, whole call: 145.5 us with a stride over
     // the grid, 142.4 us with ranges).
-    grid_wait();
-    const uint64_t total = a.ctrl->total_chunks;
+    __shared__ StatsPlan plan;
+    uint64_t total;
+    if constexpr (kOwn) {
+      total = stats_plan(plan, static_cast<const fsz_cfield*>(src), nfields, n);
+    } else {
+      grid_wait();
+      total = a.ctrl->total_chunks;
+    }
     for (uint64_t k = uint64_t(blockIdx.x) * kStatsThreads + threadIdx.x; k < kFlagStride * total;
          k += uint64_t(gridDim.x) * kStatsThreads)
       a.flags[k] = 0;  // (lookback flags, for the compression kernel)
@@ -153,10 +254,20 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
       const int seg = int(min(uint64_t(kSegChunks), gn - k0));
       if (int(threadIdx.x) < seg) {
         const uint64_t g = g0 + k0 + threadIdx.x;
-        const uint32_t f = a.chunk_field[g];
-        const FieldInfo* fi = a.fields + f;
-        const uint64_t e0 = (g - fi->chunk_first) * uint64_t(kCChunkElems);
-        s_item[threadIdx.x] = StatsItem{fi->in + e0, uint32_t(min(fi->n - e0, uint64_t(kCChunkElems))), f};
+        if constexpr (kOwn) {  // the last field that begins at or before the chunk
+          uint32_t f = 0;
+#pragma unroll
+          for (uint32_t s = kStatsPlanned / 2; s > 0; s >>= 1)
+            if (f + s < nfields && plan.first[f + s] <= g) f += s;
+          const uint64_t e0 = (g - plan.first[f]) * uint64_t(kCChunkElems);
+          s_item[threadIdx.x] =
+              StatsItem{plan.in[f] + e0, uint32_t(min(plan.n[f] - e0, uint64_t(kCChunkElems))), f};
+        } else {
+          const uint32_t f = a.chunk_field[g];
+          const FieldInfo* fi = a.fields + f;
+          const uint64_t e0 = (g - fi->chunk_first) * uint64_t(kCChunkElems);
+          s_item[threadIdx.x] = StatsItem{fi->in + e0, uint32_t(min(fi->n - e0, uint64_t(kCChunkElems))), f};
+        }
       }
       __syncthreads();
       int parts = 0;
@@ -171,51 +282,12 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
         }
       }
       __syncthreads();
+      if constexpr (kOwn) grid_wait();  // (the records are there)
       if (int(threadIdx.x) < parts) publish(int(threadIdx.x));
       __syncthreads();
     }
+    if constexpr (kOwn) grid_wait();
   }
-}
-
-// n *= dk; false if the product exceeds kMaxElems (n itself does not). Without a 64-bit
-// division, which the single thread that plans a field would wait for.
-__device__ __forceinline__ bool times_dim(uint64_t* n, uint64_t dk) {
-  if (__umul64hi(*n, dk) != 0) return false;
-  *n *= dk;
-  return *n <= kMaxElems;
-}
-
-// Validates one compression descriptor and fills the field's shape (host-visible errors
-// of the one-field entry point are checked again here for batches).
-__device__ uint32_t plan_cfield(FieldInfo* fi, const fsz_cfield& d) {
-  fi->in = d.in;
-  fi->out = static_cast<uint8_t*>(d.out);
-  fi->cap = d.out_capacity;
-  fi->out_bytes = d.out_bytes;
-  fi->mode = d.mode;
-  fi->eb_req = d.eb;
-  fi->ndim = d.dims.ndim;
-  fi->nchunks = 0;
-  fi->features_off = d.features_off;
-  if (d.dims.ndim < 1 || d.dims.ndim > 3 || d.dims.reserved != 0 || !features_valid(d.features_off) ||
-      d.mode > 1 || !(d.eb > 0.0) || isinf(d.eb) || d.out == nullptr)
-    return FSZ_ERR_INVALID_ARG;
-  uint64_t n = 1;
-  for (uint32_t k = 0; k < d.dims.ndim; ++k) {
-    const uint64_t dk = d.dims.dims[k];
-    if (!times_dim(&n, dk)) return FSZ_ERR_INVALID_ARG;
-    fi->dims[k] = dk;
-  }
-  if (n > kMaxElems) return FSZ_ERR_INVALID_ARG;
-  if ((reinterpret_cast<uintptr_t>(d.in) & 15) || (reinterpret_cast<uintptr_t>(d.out) & 15))
-    return FSZ_ERR_ALIGN;
-  if (n > 0 && d.in == nullptr) return FSZ_ERR_INVALID_ARG;
-  const uint64_t T = (n + kTile - 1) / kTile;
-  fi->n = n;
-  fi->T = T;
-  if (d.out_capacity < 64 + 8 * T) return FSZ_ERR_CAPACITY;
-  fi->nchunks = (T + kCChunkTiles - 1) / kCChunkTiles;
-  return FSZ_OK;
 }
 
 // Parses and checks a stream's preamble (the same rules as the format's definition:
@@ -481,8 +553,7 @@ __device__ __forceinline__ uint32_t field_of_chunk(const SelfPlan& S, uint32_t n
 // of waiting for its records and its chunk -> field table, unless they are so many that reading
 // every field in each costs more (whole calls behind it and for themselves: 32 fields of 258 MB
 // 62.8 / 60.5 us; 512 of 256 KB, 128 CTAs: 47.4 / 44.5; 128 of 4 MB, 608 CTAs: 105.6 / 104.6;
-// 256 of 4 MB: 193.4 / 196.3). The value-range pass of a compression does not do it: with the
-// registers and the shared memory that takes, the 32 fields went from 118.7 to 121.0 us.
+// 256 of 4 MB: 193.4 / 196.3).
 constexpr uint32_t kSelfPlanReads = 128 * 608;  // fields x CTAs
 __global__ void __launch_bounds__(kSizeThreads) fsz_sizes_kernel(KernelArgs a, const fsz_dfield* d_fields,
                                                                  uint32_t nfields, uint64_t chunk_cap) {
@@ -645,7 +716,7 @@ LaunchCfg stats_cfg() {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fsz_stats_kernel<true>, kStatsThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fsz_stats_kernel<kStatsSingle>, kStatsThreads, 0);
     LaunchCfg c;
     c.sms = sms;
     c.per = per > 0 ? per : 1;
@@ -657,13 +728,15 @@ LaunchCfg stats_cfg() {
 
 void launch_stats(const KernelArgs& a, const float* in, uint64_t n, cudaStream_t st) {
   const uint64_t chunks = (n + kCChunkElems - 1) / kCChunkElems;
-  launch_dependent(fsz_stats_kernel<true>, sched_grid(stats_cfg(), kSchedStats, chunks), kStatsThreads,
-                   0, st, a, in, n);
+  launch_dependent(fsz_stats_kernel<kStatsSingle>, sched_grid(stats_cfg(), kSchedStats, chunks),
+                   kStatsThreads, 0, st, a, static_cast<const void*>(in), n, 0u);
 }
 
-void launch_stats_batch(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st) {
-  launch_dependent(fsz_stats_kernel<false>, sched_grid(stats_cfg(), kSchedStats, max_chunks),
-                   kStatsThreads, 0, st, a, nullptr, uint64_t(0));
+void launch_stats_batch(const KernelArgs& a, const fsz_cfield* d_fields, uint32_t nfields,
+                        uint64_t chunk_cap, uint64_t max_chunks, cudaStream_t st) {
+  launch_dependent(nfields <= kStatsPlanned ? fsz_stats_kernel<kStatsBatchOwn> : fsz_stats_kernel<kStatsBatch>,
+                   sched_grid(stats_cfg(), kSchedStats, max_chunks), kStatsThreads, 0, st, a,
+                   static_cast<const void*>(d_fields), chunk_cap, nfields);
 }
 
 void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t chunk_cap, cudaStream_t st) {
