@@ -129,7 +129,7 @@ fsz_status prepare_one(const float* d_in, fsz_dims dims, fsz_eb_mode mode, doubl
   call.desc.out_bytes = d_out_bytes;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   KernelArgs a = make_args(d_ws, call.L);
-  a.early = early;
+  a.early = a.derive = early;
   launch_setup_compress(a, call.desc, call.L.chunk_cap, s);  // (clears the workspace it uses)
   if (call.desc.nchunks > 0) launch_stats(a, d_in, call.desc.n, s);
   return launched();
@@ -145,7 +145,7 @@ fsz_status encode_one(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double
                                  features_off);
   if (st != FSZ_OK || call.desc.nchunks == 0) return st;
   KernelArgs a = make_args(d_ws, call.L);
-  a.early = early;
+  a.early = a.derive = early;
   launch_compress(a, call.desc.nchunks, reinterpret_cast<cudaStream_t>(stream),
                   features_off == 0 ? kCompressFull : kCompressFeatures);
   return launched();
@@ -329,7 +329,7 @@ fsz_status fsz_compress_tiled(const float* d_in, fsz_dims dims, fsz_eb_mode mode
   call.desc.features_off = features_off | tile_word_of(int(block), int(tile_blocks));
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   KernelArgs a = make_args(d_ws, call.L);
-  a.early = true;
+  a.early = a.derive = true;
   launch_setup_compress(a, call.desc, call.L.chunk_cap, s);
   launch_stats(a, d_in, n, s);
   launch_compress_tiled(a, call.desc.nchunks, int(block), int(tile_blocks), s);
@@ -354,7 +354,8 @@ fsz_status fsz_compress_batched(const fsz_cfield* d_fields, uint32_t nfields, ui
   const WsLayout L = ws_layout(n_total / kTile + nfields, nfields);
   if (ws_bytes < L.bytes) return FSZ_ERR_WORKSPACE;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const KernelArgs a = make_args(d_ws, L);
+  KernelArgs a = make_args(d_ws, L);
+  a.early = true;
   launch_plan_compress(a, d_fields, nfields, L.chunk_cap, s);
   const uint64_t max_chunks = n_total / kCChunkElems + nfields;
   launch_stats_batch(a, d_fields, nfields, L.chunk_cap, max_chunks, s);

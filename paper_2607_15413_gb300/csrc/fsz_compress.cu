@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
   uint64_t total = 0;
   uint32_t group = 1, lead = 1, seq_t = 0, end_seq = kNone;
   bool single = true;
-  float step_s = 0.0f, step_r = 0.0f;  // a.early: the field's step (lane 0), 0 if it is refused
+  float step_s = 0.0f, step_r = 0.0f;  // a.derive: the field's step (lane 0), 0 if it is refused
   auto launch_tickets = [&](uint64_t chunks) {
     total = chunks;
     group = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
@@ -567,14 +567,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
           ci.flags = kInfoEnd;
         } else {
           // (from L2 before grid_wait: L1 may hold an earlier call's record)
-          FieldInfo* fi = single ? a.fields : a.fields + a.chunk_field[c];
           const auto get = [&](const auto* p) { return early ? __ldcg(p) : *p; };
+          FieldInfo* fi = single ? a.fields : a.fields + get(a.chunk_field + c);
           const uint64_t first = get(&fi->chunk_first), T = get(&fi->T), n = get(&fi->n);
           const uint64_t nchunks = get(&fi->nchunks), cap = get(&fi->cap);
           const uint64_t in = get(reinterpret_cast<const uint64_t*>(&fi->in));
           const uint64_t out = get(reinterpret_cast<const uint64_t*>(&fi->out));
           const uint32_t off = get(&fi->features_off);
-          const float s = early ? 1.0f : a.early ? step_s : fi->s, r = a.early ? step_r : fi->r;
+          const float s = early ? 1.0f : a.derive ? step_s : fi->s, r = early || a.derive ? step_r : fi->r;
           const uint64_t lc = c - first;
           const uint64_t tile0 = lc * Cfg::kChunkTiles;
           const uint64_t e0 = lc * kCChunkElems;
@@ -617,11 +617,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     }
   };
 
-  // A one-field call (a.early): the value-range pass releases this kernel once the set-up
-  // kernel before it has completed, so the first ticket is taken and its quads are loaded
-  // under the end of that pass; only the step is missing (31 MB field 26.9 -> 25.4 us).
+  // Right behind its value-range pass (a.early): the pass releases this kernel once the set-up or
+  // planning kernel before it has completed, so the first ticket is taken and its quads are
+  // loaded under the end of that pass; only the step is missing (31 MB field 26.9 -> 25.4 us; a
+  // batch of 32 mixed fields of 258 MB 118.7 -> 116.9, of 8 fields of 256 KB 13.2 -> 11.7).
   if (a.early) {
     if (warp == kHostWarp) {
+      single = __ldcg(&a.ctrl->nfields) == 1;
       launch_tickets(__ldcg(&a.ctrl->total_chunks));
       take_ticket(true);
     } else if (warp < kWarps) {
@@ -629,7 +631,18 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     }
   }
   grid_wait();
-  if (a.early && warp == kHostWarp && lane == 0) {
+  if (a.early && !a.derive && warp == kHostWarp && lane == 0) {
+    for (uint32_t k = 0; k < seq_t; ++k) {
+      ChunkInfo& ci = S.meta[k];
+      if (ci.flags & kInfoEnd) continue;
+      ci.r = __ldcg(&ci.fi->r);
+      if (!(__ldcg(&ci.fi->s) > 0.0f)) {
+        ci.cnt = 0;
+        ci.flags &= ~kInfoOk;
+      }
+    }
+  }
+  if (a.derive && warp == kHostWarp && lane == 0) {
     // Each CTA derives the step for itself: the value-range pass need not find its last CTA and
     // wait for it, nor this one for the record (31 MB field 24.9 -> 23.7 us, 2^20 values equal). The CTA
     // with the first chunk records it.
@@ -700,7 +713,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
               uint8_t* const base = ci.out + ci.data_base + excl;
               place_runs<kResolverRuns, kWarps - kResolverRuns>(S, b, base, lane);
               if (lane == 0 && (ci.flags & kInfoLast))
-                write_preamble(ci.fi, excl + tot, a.early ? step_s : ci.fi->s, Cfg::kT);
+                write_preamble(ci.fi, excl + tot, a.derive ? step_s : ci.fi->s, Cfg::kT);
             }
           }
           // the runs are read: their ring space goes back to the compute warps

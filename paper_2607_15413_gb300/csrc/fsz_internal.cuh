@@ -170,9 +170,10 @@ struct KernelArgs {
   uint64_t* flags;       // compression: lookback flags
   uint32_t* sums;        // decompression: payload bytes of each chunk,
   uint32_t* block_sums;  // ... and of each kSumBlock consecutive ones
-  // compression of one field: the compression kernel starts under the value-range pass and
+  // compression: the compression kernel starts under the value-range pass; for one field it
   // derives the step itself
   bool early = false;
+  bool derive = false;
   uint64_t skip_chunk;  // test hook: this chunk publishes no flag (decompression: no record)
   uint64_t timeout_ns;  // bound on every spin-wait
   // multipass compression only: the four variants' tile costs, variant-major (given_T

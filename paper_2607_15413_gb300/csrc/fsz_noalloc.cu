@@ -102,7 +102,7 @@ extern "C" fsz_status fsz_compress_noalloc(const float* d_in, fsz_dims dims, fsz
   a.fields = reinterpret_cast<FieldInfo*>(base + L.fields_off);
   a.chunk_field = reinterpret_cast<const uint32_t*>(base + L.map_off);
   a.flags = reinterpret_cast<uint64_t*>(base + L.flags_off);
-  a.early = true;
+  a.early = a.derive = true;
   a.skip_chunk = ~uint64_t(0);
   a.timeout_ns = kDefaultTimeoutNs;
   launch_setup_compress(a, desc, L.chunk_cap, s);

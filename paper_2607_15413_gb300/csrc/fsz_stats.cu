@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
       atomicMax(&fi->max_key, float_key(h));
     }
     atomicMax(&fi->max_abs_bits, m);
-    if (kSingle && a.early) return;  // (the compression kernel behind this one derives the step)
+    if (kSingle && a.derive) return;  // (the compression kernel behind this one derives the step)
     __threadfence();
     const uint32_t prev = atomicAdd(&fi->done_chunks, s_cnt[k]);
     if (uint64_t(prev) + s_cnt[k] == fi->nchunks) {
@@ -283,10 +283,12 @@ __global__ void __launch_bounds__(kStatsThreads, 5) fsz_stats_kernel(KernelArgs 
       }
       __syncthreads();
       if constexpr (kOwn) grid_wait();  // (the records are there)
+      if (k0 + kSegChunks >= gn) grid_release();  // (the compression kernel may take its first tickets)
       if (int(threadIdx.x) < parts) publish(int(threadIdx.x));
       __syncthreads();
     }
     if constexpr (kOwn) grid_wait();
+    grid_release();
   }
 }
 

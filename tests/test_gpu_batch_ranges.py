@@ -83,3 +83,37 @@ def test_ranges_of_several_segments(fszlib):
     for k, x in enumerate(xs):
         ref, nb = fszlib.compress(x, 1e-3)
         assert ks[k] == nb and torch.equal(b.stream(k, ks), ref)
+
+
+@pytest.mark.parametrize("nfields", [3, 64, 65, 200])
+def test_fields_refused_in_one_call_and_not_in_the_next(fszlib, nfields):
+    """Queued without waits: the compression kernel takes its first chunks before their fields' steps
+    are known."""
+    dev = _cuda()
+    good = [torch.from_numpy(inputs.sinusoids(20000 + 7 * k, seed=k % 5)).to(dev) for k in range(nfields)]
+    xs = [x.clone() for x in good]
+    b = fszlib.CompressBatch([(x, (x.numel(),), fszlib.EB_REL, 1e-3) for x in xs], device=dev)
+    sizes, arenas, statuses = [], [], []
+    torch.cuda.synchronize()
+    for call in range(4):
+        for k in range(nfields):
+            xs[k].copy_(good[k])
+            if (k + call) % 3 == 0:
+                xs[k][11 * call + k] = float("nan")
+        b.arena.fill_(0xA5)
+        b.sizes.zero_()
+        assert b.run() == fszlib.OK
+        sizes.append(b.sizes.clone())
+        arenas.append(b.arena.clone())
+        if call == 3:
+            statuses = b.status()[1]
+    refs = [fszlib.compress(x, 1e-3)[0] for x in good]
+    for call in range(4):
+        ks = sizes[call].tolist()
+        for k in range(nfields):
+            slot = arenas[call][b.offsets[k]:b.offsets[k] + b.caps[k]]
+            if (k + call) % 3 == 0:
+                assert ks[k] == 0
+            else:
+                assert ks[k] == refs[k].numel() and torch.equal(slot[:ks[k]], refs[k]), (call, k)
+    assert statuses == [fszlib.ERR_NONFINITE if (k + 3) % 3 == 0 else fszlib.OK for k in range(nfields)]
