@@ -101,7 +101,8 @@ static_assert(kWarps <= 32, "one lane per quad in the chunk scan");
 // instead of two fences around one took the kernel from 147 to 141 us at 512^3.)
 constexpr uint32_t kInfoOk = 1u, kInfoLast = 2u, kInfoFirst = 4u, kInfoSkip = 8u, kInfoEnd = 16u;
 struct __align__(16) ChunkInfo {
-  uint32_t cnt;          // elements to load: the chunk's, or 0 (a refused field, the end)
+  uint32_t cnt;          // elements to load: the chunk's, or 0 (a field known to be refused, the
+                         // end); not changed once the slot is handed over
   uint32_t ntiles;
   float r;
   uint32_t flags;        // kInfo* bits; kInfoEnd: no chunk, the CTA's chunks have run out
@@ -620,7 +621,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
   // Right behind its value-range pass (a.early): the pass releases this kernel once the set-up or
   // planning kernel before it has completed, so the first ticket is taken and its quads are
   // loaded under the end of that pass; only the step is missing (31 MB field 26.9 -> 25.4 us; a
-  // batch of 32 mixed fields of 258 MB 118.7 -> 116.9, of 8 fields of 256 KB 13.2 -> 11.7).
+  // batch of 32 mixed fields of 258 MB 118.7 -> 116.9, of 8 fields of 256 KB 13.2 -> 11.7). A field
+  // that turns out to be refused only loses kInfoOk: its count stays, so that load_first() and the
+  // main loop agree on which chunks have been loaded, and the loop waits for every one of them
+  // before it loads the next chunk (of another field, perhaps) into the same buffer.
   if (a.early) {
     if (warp == kHostWarp) {
       single = __ldcg(&a.ctrl->nfields) == 1;
@@ -636,10 +640,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
       ChunkInfo& ci = S.meta[k];
       if (ci.flags & kInfoEnd) continue;
       ci.r = __ldcg(&ci.fi->r);
-      if (!(__ldcg(&ci.fi->s) > 0.0f)) {
-        ci.cnt = 0;
-        ci.flags &= ~kInfoOk;
-      }
+      if (!(__ldcg(&ci.fi->s) > 0.0f)) ci.flags &= ~kInfoOk;
     }
   }
   if (a.derive && warp == kHostWarp && lane == 0) {
@@ -662,10 +663,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     for (uint32_t k = 0; k < seq_t; ++k) {
       ChunkInfo& ci = S.meta[k];
       ci.r = step_r;
-      if (st != FSZ_OK) {
-        ci.cnt = 0;
-        ci.flags &= ~kInfoOk;
-      }
+      if (st != FSZ_OK) ci.flags &= ~kInfoOk;
       if (ci.flags & kInfoFirst) {
         if (st == FSZ_OK)
           store_step(a.fields, p);
@@ -816,9 +814,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     const ChunkInfo& ci = S.meta[b];
     const uint32_t flags = ci.flags;
     const bool end = (flags & kInfoEnd) != 0;
-    const uint32_t qv = quad_valid(ci.cnt);
+    const bool loaded = quad_valid(ci.cnt) != 0;
     float d[32];
-    if (qv) {
+    if (loaded) {
       cp_async_wait_all();
       __syncwarp();
       // lane L reads block g = L & 7 of tile L >> 3: piece k at column k ^ g of its row
@@ -833,7 +831,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     uint32_t qlen = 0;
     QuadPlan P;
     const int qt0 = Cfg::kQuadTiles * warp;            // the quad's first tile in the chunk
-    const bool any = qv != 0;
+    const bool any = loaded && (flags & kInfoOk);  // (a refused field's quad is dropped)
     if (any) {
       const int t = qt0 + lane / Cfg::kLanes;
       const bool live = t < int(ci.ntiles);
