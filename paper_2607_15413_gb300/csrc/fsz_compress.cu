@@ -365,9 +365,15 @@ __device__ __forceinline__ void plan_quad(const float (&d)[32], const float r, c
     A += __shfl_xor_sync(FULL, A, o);
     B += __shfl_xor_sync(FULL, B, o);
   }
+  // The partial sums of a tile of more than 256 elements can overflow with both signs (|d| < 2^120.5,
+  // by the step's cap), which leaves no mean: the maxima above drop the NaN, and the variant would
+  // seem to save block 0's first residual. It is ruled out here. (128 elements' sums are finite, so
+  // a smaller tile's mean is a number or infinite, and an infinite one has the highest cost.)
+  int penc = pen3;
+  if constexpr (Cfg::kElems > 256) penc = fabsf(muY) < 2.0f * kMagBase ? pen3 : 0x10000;
   int C1 = int(A & 0xffffu), C2 = int(A >> 16);
-  int C3 = 4 + int(B & 0xffffu) + pen3;
-  int C4 = 4 + int(B >> 16) + pen2 + pen3;
+  int C3 = 4 + int(B & 0xffffu) + penc;
+  int C4 = 4 + int(B >> 16) + pen2 + penc;
   if constexpr (kGiven) {
     C1 = int(given[0]);
     C2 = int(given[gT]);
