@@ -861,6 +861,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
     last = __shfl_sync(FULL, last, 0);
     if (last) {
       if (!end) {
+        __syncwarp();  // lane 0's acquire (the other warps' lengths) before every lane's reads
         const uint32_t ql = lane < kWarps ? S.qlen[b][lane] : 0u;
         uint32_t inc = ql;
 #pragma unroll
