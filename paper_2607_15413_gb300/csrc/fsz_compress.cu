@@ -573,7 +573,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) fsz_compress_kernel(Kern
           ci.cnt = 0;
           ci.flags = kInfoEnd;
         } else {
-          // (from L2 before grid_wait: L1 may hold an earlier call's record)
+          // (early, the value-range pass is still writing other words of the record's lines: from
+          // L2, so that no half-written line is in L1)
           const auto get = [&](const auto* p) { return early ? __ldcg(p) : *p; };
           FieldInfo* fi = single ? a.fields : a.fields + get(a.chunk_field + c);
           const uint64_t first = get(&fi->chunk_first), T = get(&fi->T), n = get(&fi->n);

@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_sizes_kernel(KernelArgs a, c
     grid_wait();
     total = a.ctrl->total_chunks;
   }
-  grid_release();
+  grid_release();  // (the records may not be there yet: the successor loads nothing early)
   for (uint64_t b = blockIdx.x; b * kSumBlock < total; b += gridDim.x) {
     uint32_t bytes[kChunksPerWarp];
 #pragma unroll
