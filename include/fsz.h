@@ -198,7 +198,9 @@ fsz_status fsz_compress_tiled(const float* d_in, fsz_dims dims, fsz_eb_mode mode
                               uint32_t block, uint32_t tile_blocks, uint32_t features_off,
                               void* d_out, uint64_t out_capacity, uint64_t* d_out_bytes, void* d_ws,
                               uint64_t ws_bytes, fsz_stream stream);
-/* Decodes a stream of any tile configuration (including the default). */
+/* Decodes a stream of any tile configuration (including the default). The rate headers are
+ * checked first: a stream that is refused for its preamble, a malformed header or sizes that do
+ * not add up leaves d_out as it was (only a malformed mean is met while decoding). */
 fsz_status fsz_decompress_tiled(const void* d_in, uint64_t in_bytes, float* d_out,
                                 uint64_t out_capacity_elems, void* d_ws, uint64_t ws_bytes,
                                 fsz_stream stream);

@@ -166,6 +166,10 @@ fsz_status decompress_one(const void* d_in, uint64_t in_bytes, float* d_out,
   a.in_bytes = in_bytes;
   a.dout = d_out;
   a.cap_elems = out_capacity_elems;
+  if (kind == kDecompressTiled) {
+    a.found = reinterpret_cast<uint64_t*>(const_cast<uint32_t*>(a.chunk_field));
+    a.nfound = uint32_t(setup_decompress_grid(out_capacity_elems));
+  }
   launch_setup_decompress(a, L.chunk_cap, s, kind == kDecompressTiled);
   launch_decompress(a, (out_capacity_elems + kDChunkElems - 1) / kDChunkElems, s, kind);
   return launched();

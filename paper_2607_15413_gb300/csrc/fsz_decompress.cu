@@ -101,12 +101,6 @@ __device__ __forceinline__ uint64_t block_word_offsets(uint64_t h) {
   return (W * 0x0101010101010101ULL) << 8;
 }
 
-// A byte that begins a tile reserves bit 5 (bits 7 and 6 are its flags), the others bits 5-7.
-__device__ __forceinline__ bool header_reserved_bits_set(uint64_t h, int T, uint64_t unit) {
-  const uint64_t flags = 3 * unit_centring_bits(T, unit);  // 0x40 and 0x80
-  return (h & (0xE0E0E0E0E0E0E0E0ULL & ~flags)) != 0;
-}
-
 // *p if `in`, else 0, read here: a plain load is moved down to its use by the compiler, past
 // the work that it is meant to run under. ld_now32 reads from L2.
 __device__ __forceinline__ uint64_t ld_now(const void* p, bool in) {
@@ -362,8 +356,9 @@ __device__ __forceinline__ Field field_of_stream(const KernelArgs& a) {
 // kAny: also decodes streams without the cross-block state. kPrezero: the output already
 // holds zeros; tiles whose 8 blocks all have rate 0 and no mean (all +0.0) are neither
 // decoded nor written (the adaptive pre-zero of Sec. 3.1 for high compression ratios).
-// Cfg: the tile configuration.
-template <bool kAny, bool kPrezero, typename Cfg>
+// Cfg: the tile configuration. kChecked: a tiled call, whose set-up kernel has checked every rate
+// header; nothing is decoded if it found one malformed, or sizes that do not add up to the data's.
+template <bool kAny, bool kPrezero, bool kChecked, typename Cfg>
 __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
   DecompressSmem& S = *reinterpret_cast<DecompressSmem*>(smem_raw);
@@ -471,7 +466,7 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
     fetch_sizes();
     if (verdict == 0) nt = 0;
     total = verdict;
-    const uint32_t off_bits = ((f.features_off & kOffLz2) ? 2u : 0u) | ((f.features_off & kOffCenter) ? 1u : 0u);
+    const uint32_t off_bits = forbidden_flags(f.features_off);
     uint32_t r0 = 0;  // the group's first record: seq % recs
     for (uint32_t seq = 0;;) {
       uint32_t next = 0;
@@ -503,9 +498,7 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
       // cross-block state are decoded by the kAny instance only
       const bool unsupported = !kAny && (f.features_off & kOffCross) && nt > 0;
       if (unsupported) set_error(a.ctrl, a.fields + fidx, FSZ_ERR_INVALID_ARG);
-      const uint32_t forbid =
-          single ? off_bits
-                 : ((f.features_off & kOffLz2) ? 2u : 0u) | ((f.features_off & kOffCenter) ? 1u : 0u);
+      const uint32_t forbid = single ? off_bits : forbidden_flags(f.features_off);
       const bool any_forbid = __any_sync(FULL, forbid != 0);
       uint32_t bad = 0;
 #pragma unroll
@@ -587,6 +580,18 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
     // order, so the bytes in use are head - freed; pos is head's place in the ring.
     uint32_t head = 0, freed = 0, pos = 0;
     uint32_t oldest = 0;  // the oldest chunk whose bytes are not yet known to be released
+    // A tiled call's rate headers as the set-up kernel found them (here, where it costs nothing: the
+    // first record is still being made; in the header warp it cost 1 us of 23).
+    uint64_t headers = 0;
+    if constexpr (kChecked) {
+      bool malformed = false;
+      for (uint32_t k = lane; k < a.nfound; k += 32) {
+        const uint64_t found = __ldcg(reinterpret_cast<const unsigned long long*>(a.found) + k);
+        malformed |= found == kHeadersBad;
+        headers += found;
+      }
+      headers = __any_sync(FULL, malformed) ? kHeadersBad : warp_sum_u64(headers);
+    }
     for (uint32_t seq = 0;; ++seq) {
       const int r = int(seq % recs);
       if (!mbar_wait(&S.fetched[r], (seq / recs) & 1u, wait_ns)) {
@@ -604,6 +609,7 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
       bool valid = q.bad == 0;
       if (q.data_base + excl + tot > q.in_bytes) valid = false;
       if (q.last && excl + tot != q.data_bytes) valid = false;
+      if (kChecked && headers != q.data_bytes) valid = false;
       const uint64_t base = reinterpret_cast<uint64_t>(q.sin);
       const uint64_t src = base + q.data_base + excl;
       const uint64_t a0 = src & ~uint64_t(15);
@@ -766,7 +772,7 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
 
 template <bool kAny, bool kPrezero>
 __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_kernel(KernelArgs a) {
-  decompress_cta<kAny, kPrezero, DefaultCfg>(a);
+  decompress_cta<kAny, kPrezero, false, DefaultCfg>(a);
 }
 
 // Any tile configuration: the stream's own, from its preamble (a configuration that does not
@@ -778,13 +784,13 @@ __global__ void __launch_bounds__(kThreads, 2) fsz_decompress_tiled_kernel(Kerne
   int B = 32, T = 8;
   if (a.in_bytes < 64 || !config_of(*reinterpret_cast<const uint32_t*>(a.sin + 52), &B, &T)) B = 32, T = 8;
   if (B == 32) {
-    if (T == 4) decompress_cta<true, false, TileCfg<32, 4>>(a);
-    else if (T == 8) decompress_cta<true, false, TileCfg<32, 8>>(a);
-    else decompress_cta<true, false, TileCfg<32, 16>>(a);
+    if (T == 4) decompress_cta<true, false, true, TileCfg<32, 4>>(a);
+    else if (T == 8) decompress_cta<true, false, true, TileCfg<32, 8>>(a);
+    else decompress_cta<true, false, true, TileCfg<32, 16>>(a);
   } else {
-    if (T == 4) decompress_cta<true, false, TileCfg<64, 4>>(a);
-    else if (T == 8) decompress_cta<true, false, TileCfg<64, 8>>(a);
-    else decompress_cta<true, false, TileCfg<64, 16>>(a);
+    if (T == 4) decompress_cta<true, false, true, TileCfg<64, 4>>(a);
+    else if (T == 8) decompress_cta<true, false, true, TileCfg<64, 8>>(a);
+    else decompress_cta<true, false, true, TileCfg<64, 16>>(a);
   }
 }
 

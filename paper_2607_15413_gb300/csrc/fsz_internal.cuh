@@ -146,8 +146,11 @@ struct alignas(64) Ctrl {
 
 // Workspace layout: [Ctrl][FieldInfo x nfields][u32 chunk->field x cap][u64 flags x cap].
 // Decompression keeps its chunks' payload sizes (u32 x cap, and one sum per kSumBlock
-// chunks) where compression keeps its lookback flags.
+// chunks) where compression keeps its lookback flags; a tiled decompression, which has one field
+// and so no table, keeps what its set-up kernel found (u64 x one per kSumBlock chunks at most)
+// where batches keep the table.
 constexpr int kSumBlock = 32;
+constexpr uint64_t kHeadersBad = uint64_t(1) << 63;
 struct WsLayout {
   uint64_t fields_off, map_off, flags_off, bytes;
   uint64_t chunk_cap;
@@ -186,6 +189,10 @@ struct KernelArgs {
   uint64_t in_bytes = 0;
   float* dout = nullptr;
   uint64_t cap_elems = 0;
+  // a tiled call: what each of the set-up kernel's CTAs found in its part of the rate headers
+  // (kHeadersBad, or the payload bytes that they give)
+  uint64_t* found = nullptr;
+  uint32_t nfound = 0;
   // work assignment (from the schedule, set by the launch functions)
   uint32_t ticket_chunks = 1;  // consecutive chunks per ticket
   uint32_t ticket_lead = 1;    // compression: tickets taken ahead of the compute warps
@@ -563,6 +570,18 @@ __device__ __forceinline__ uint32_t unit_bytes(uint64_t h, int B, int T, uint64_
   return uint32_t(B / 8) * words + 4u * uint32_t(__popcll(h & unit_centring_bits(T, unit)));
 }
 
+// A byte that begins a tile reserves bit 5 (bits 7 and 6 are its flags), the others bits 5-7.
+__device__ __forceinline__ bool header_reserved_bits_set(uint64_t h, int T, uint64_t unit) {
+  const uint64_t flags = 3 * unit_centring_bits(T, unit);  // 0x40 and 0x80
+  return (h & (0xE0E0E0E0E0E0E0E0ULL & ~flags)) != 0;
+}
+
+// The tile flags that a stream with these features switched off may not use: unit_centring_bits()
+// times 2 (second order) and 1 (centred).
+__device__ __forceinline__ uint32_t forbidden_flags(uint32_t features_off) {
+  return ((features_off & kOffLz2) ? 2u : 0u) | ((features_off & kOffCenter) ? 1u : 0u);
+}
+
 // ------------------------------------------------------------------ float keys
 
 __device__ __forceinline__ uint32_t float_key(float x) {
@@ -781,7 +800,8 @@ void launch_decompress(const KernelArgs& a, uint64_t max_chunks, cudaStream_t st
 // clears the lookback flags, for decompression it sizes the chunks' payloads (no memset of
 // the workspace needed). launch_sizes: the sizing of a batch behind its planning kernel.
 void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t chunk_cap, cudaStream_t st);
-// tiled: any tile configuration's stream (of at most max_chunks chunks).
+// tiled: any tile configuration's stream; a.nfound is then setup_decompress_grid.
+int setup_decompress_grid(uint64_t cap_elems);
 void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st,
                              bool tiled = false);
 void launch_sizes(const KernelArgs& a, const fsz_dfield* d_fields, uint32_t nfields, uint64_t chunk_cap,

@@ -414,8 +414,8 @@ constexpr int kSizeThreads = 32 * kSizeWarps;
 constexpr int kChunksPerWarp = kSumBlock / kSizeWarps;  // of a block: warp, warp + kSizeWarps
 
 // Records the sizes of one block of chunks; bytes[k]: this lane's unit of chunk
-// kSumBlock * block + kSizeWarps * k + warp (0 beyond the last one).
-__device__ __forceinline__ void write_chunk_sizes(const KernelArgs& a, uint64_t block, uint64_t total,
+// kSumBlock * block + kSizeWarps * k + warp (0 beyond the last one). Returns their sum in thread 0.
+__device__ __forceinline__ uint32_t write_chunk_sizes(const KernelArgs& a, uint64_t block, uint64_t total,
                                                   const uint32_t (&bytes)[kChunksPerWarp],
                                                   uint32_t* s_sum) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -429,17 +429,21 @@ __device__ __forceinline__ void write_chunk_sizes(const KernelArgs& a, uint64_t 
     }
   }
   __syncthreads();
+  uint32_t all = 0;
   if (warp == 0) {
-    const uint32_t sum = __reduce_add_sync(0xffffffffu, s_sum[lane]);
-    if (lane == 0) a.block_sums[block] = sum;
+    all = __reduce_add_sync(0xffffffffu, s_sum[lane]);
+    if (lane == 0) a.block_sums[block] = all;
   }
   __syncthreads();
+  return all;
 }
 
 // One field: sized beside the parsing of its preamble (by one thread of CTA 0) rather than
 // after it. The element count is read from the preamble as it stands, bounded by the
 // output's capacity, and the headers within the stream's buffer; the sizes of a stream that
-// the parsing refuses are not used.
+// the parsing refuses are not used. kTiled: the headers are checked too, and what each CTA found
+// left for the decompression kernel, which writes nothing for a stream whose headers are malformed
+// or do not add up to its data.
 template <bool kTiled>
 __global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(KernelArgs a,
                                                                             uint64_t chunk_cap) {
@@ -453,8 +457,11 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(Kern
   const uint64_t n = in_bytes >= 64 ? *reinterpret_cast<const uint64_t*>(in + 8) : 0;
   const uint64_t room = in_bytes >= 64 ? in_bytes - 64 : 0;  // bytes after the preamble
   int B = 32, TB = 8;
+  uint64_t forbid = 0;
   if constexpr (kTiled) {
-    if (in_bytes >= 64 && !config_of(*reinterpret_cast<const uint32_t*>(in + 52), &B, &TB)) B = 32, TB = 8;
+    const uint32_t word = in_bytes >= 64 ? *reinterpret_cast<const uint32_t*>(in + 52) : 0u;
+    if (!config_of(word, &B, &TB)) B = 32, TB = 8;
+    forbid = forbidden_flags(word);
   }
   // rate bytes 8 (u + 0 .. 7), or as many of them as there are before `end`
   auto load_unit = [&](uint64_t u, uint64_t end) -> uint64_t {
@@ -488,6 +495,8 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(Kern
   const uint64_t nc = min(n, cap_elems);
   const uint64_t total = (nc + kDChunkElems - 1) / kDChunkElems;  // <= chunk_cap
   const uint64_t hdr_bytes = min(((nc + B * TB - 1) >> (31 - __clz(B * TB))) * TB, room);
+  uint64_t sum = 0;
+  bool bad = false;
   for (uint64_t b = blockIdx.x; b * kSumBlock < total; b += gridDim.x) {
     uint32_t bytes[kChunksPerWarp];
 #pragma unroll
@@ -496,8 +505,14 @@ __global__ void __launch_bounds__(kSizeThreads) fsz_setup_decompress_kernel(Kern
       const bool mine = uint32_t(lane) < units && 8 * u < hdr_bytes;
       if (kTiled || b != blockIdx.x) h[k] = mine ? load_unit(u, hdr_bytes) : 0;
       bytes[k] = mine ? unit_bytes(h[k], B, TB, u) : 0u;
+      if (kTiled && mine)
+        bad |= header_reserved_bits_set(h[k], TB, u) || (h[k] & (forbid * unit_centring_bits(TB, u))) != 0;
     }
-    write_chunk_sizes(a, b, total, bytes, s_sum);
+    sum += write_chunk_sizes(a, b, total, bytes, s_sum);
+  }
+  if constexpr (kTiled) {
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) a.found[blockIdx.x] = bad ? kHeadersBad : sum;
   }
 }
 
@@ -746,10 +761,13 @@ void launch_setup_compress(const KernelArgs& a, const FieldInfo& fi, uint64_t ch
   launch_dependent(fsz_setup_compress_kernel, setup_grid(nflags), kSetupThreads, 0, st, a, fi, nflags);
 }
 
+int setup_decompress_grid(uint64_t cap_elems) {
+  return sizes_grid((cap_elems + kDChunkElems - 1) / kDChunkElems);
+}
+
 void launch_setup_decompress(const KernelArgs& a, uint64_t chunk_cap, cudaStream_t st, bool tiled) {
   launch_dependent(tiled ? fsz_setup_decompress_kernel<true> : fsz_setup_decompress_kernel<false>,
-                   sizes_grid((a.cap_elems + kDChunkElems - 1) / kDChunkElems), kSizeThreads, 0, st, a,
-                   chunk_cap);
+                   setup_decompress_grid(a.cap_elems), kSizeThreads, 0, st, a, chunk_cap);
 }
 
 void launch_sizes(const KernelArgs& a, const fsz_dfield* d_fields, uint32_t nfields, uint64_t chunk_cap,
