@@ -279,17 +279,19 @@ fsz_status fsz_get_schedule_limits(uint32_t* stats_max, uint32_t* compress_max,
  * mapping; none of it changes a stream). The persistent kernels hand out work by atomic
  * tickets; a ticket covers `*_ticket_chunks` consecutive chunks of 32 tiles (1-4), the
  * unit of work a CTA takes; in each of its chunks after the first the chunk's byte offset
- * follows from the previous one (without a lookback in compression, Sec. 4.4). Compression takes
- * tickets up to `compress_ticket_lead` chunks (1-3) ahead of its compute warps;
+ * follows from the previous one (without a lookback in compression, Sec. 4.4). Compression
+ * takes tickets up to `compress_ticket_lead` chunks (1-3) ahead of its compute warps;
  * decompression keeps up to `decompress_records` chunks (2 x ticket chunks .. 16) between
- * ticket and decode per CTA (near a launch's end at most 6, by tickets of at most 2). A launch whose chunks would give fewer than
+ * ticket and decode per CTA. A launch whose chunks would give fewer than
  * `min_tickets_per_cta` tickets per CTA (0-64) at the requested ticket size takes tickets
- * of fewer chunks (down to 1), so that small fields and small batches still spread over
- * every CTA; 0 keeps the requested size at every launch size. Defaults: CTAs 0 (as many
- * as fit), compression 2 chunks per ticket with lead 2, decompression 4 chunks per ticket
- * and 16 records, 4 tickets per CTA. Read by every later call of this process at launch
- * (a CUDA graph keeps the schedule it was captured with). Used by the autotuner; not
- * thread-safe. */
+ * of fewer chunks (down to 1), compression then with lead 1, and decompression's last 16
+ * chunks per CTA (a whole launch, up to about 40 M values) are taken by tickets of at most
+ * 2 chunks with at most 6 held, so that small fields, small batches and a launch's end
+ * spread over every CTA; 0 keeps all that is requested, at every launch size and to its
+ * end. Defaults: CTAs 0 (as many as fit), compression 2 chunks per ticket with lead 2,
+ * decompression 4 chunks per ticket and 16 records, 4 tickets per CTA. Read by every later
+ * call of this process at launch (a CUDA graph keeps the schedule it was captured with).
+ * Used by the autotuner; not thread-safe. */
 typedef struct fsz_schedule {
   uint32_t stats_ctas_per_sm;
   uint32_t compress_ctas_per_sm;

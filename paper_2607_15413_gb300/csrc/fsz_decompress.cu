@@ -54,6 +54,7 @@ constexpr uint32_t kNoneChunk = 0xffffffffu;
 // to 16 chunks (30 us) held each the CTAs finished far apart. 512^3: 112.6 us without, 109.8
 // from the last 8 chunks on, 106.9 from 16, 106.2 from 32; batch of 32 fields 69.7, 66.0, 66.5,
 // 67.6 us; with kTailAhead 4 or 8: 106.8, 108.9 and 67.9, 67.0 us.
+// (A schedule whose min_tickets is 0 keeps its tickets and records to the end.)
 constexpr uint32_t kTailChunks = 16, kTailTicket = 2, kTailAhead = 6;
 
 // A chunk's header and parameters, from the header warp to the loader and the decode
@@ -409,6 +410,7 @@ __device__ __forceinline__ void decompress_cta(const KernelArgs& a) {
     auto launch_tickets = [&]() {
       full = launch_ticket_chunks(a.ticket_chunks, a.min_tickets, total, gridDim.x);
       nbig = total > gridDim.x * kTailChunks ? (total - gridDim.x * kTailChunks) / full : 0;
+      if (a.min_tickets == 0) nbig = (total + full - 1) / full;
     };
     auto place = [&](uint32_t t) {
       const bool big = t < nbig;
