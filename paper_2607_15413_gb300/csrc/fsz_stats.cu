@@ -70,11 +70,15 @@ __device__ uint32_t plan_cfield(FieldInfo* fi, const fsz_cfield& d) {
 // The chunk ranges of a batch of up to kStatsPlanned fields, worked out from the descriptors by
 // each CTA of the value-range kernel for itself: its loads then run under the planning kernel (4 to
 // 5 us of loads that wait for one another in one CTA), which only the publication of the ranges
-// waits for. An instance of its own and no more fields, because 760 CTAs of 48 registers stream
-// at the copy peak only while the L1 has room for what they have in flight. Whole calls, behind
-// the planning kernel and for themselves: 8 fields of 256 KB 14.6 / 13.3 us, 32 of 512 KB
-// 20.2 / 18.3, 32 of 8 MB 108.9 / 107.4, 64 of 8 MB 211.3 / 207.7, 32 mixed ones of 258 MB in
-// all 118.9 / 118.9; with up to 256 fields, in one instance with the other way: 121.0.
+// waits for. An instance of its own, because 760 CTAs of 48 registers stream at the copy peak only
+// while the L1 has room for what they have in flight: with up to 256 fields in one instance with
+// the other way, 32 mixed fields of 258 MB took 121.0 us instead of 118.9. Whole calls, behind the
+// planning kernel and for themselves: 32 fields of 512 KB 18.4 / 16.5 us, 64 of 256 KB 19.6 / 17.6,
+// 64 of 4 MB 108.8 / 106.1. Above 64 fields (this instance with room for 256, 6 KB of shared
+// memory) it depends on their size, for better and worse: 65 of 256 KB 20.1 / 18.0, 128 of 64 KB
+// 18.3 / 16.7, 128 of 256 KB 26.1 / 26.4, 128 of 1 MB 60.4 / 62.0, 128 of 4 MB 210.5 / 205.9, 256 of
+// 64 KB 23.8 / 24.6, 256 of 1 MB 112.2 / 107.9, 256 of 4 MB 413.6 / 407.0; so the rule on the count
+// stops where it has been better at every size.
 constexpr uint32_t kStatsPlanned = 64;
 struct StatsPlan {
   uint64_t total;
