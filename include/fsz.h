@@ -122,7 +122,8 @@ uint64_t fsz_batch_workspace_bytes(uint64_t n_total, uint32_t nfields);
  * (min, max, finiteness, and the step derived from them), then the single-pass
  * compression kernel. Writes the stream to d_out and its size to *d_out_bytes
  * (device u64, may be NULL). out_capacity must be at least 64 + 8T; a stream that
- * would exceed it sets FSZ_ERR_CAPACITY in the workspace status. */
+ * would exceed it sets FSZ_ERR_CAPACITY in the workspace status (without a preamble or a
+ * size; other bytes of d_out within its capacity may have been written). */
 fsz_status fsz_compress(const float* d_in, fsz_dims dims, fsz_eb_mode mode, double eb,
                         void* d_out, uint64_t out_capacity, uint64_t* d_out_bytes,
                         void* d_ws, uint64_t ws_bytes, fsz_stream stream);
@@ -159,7 +160,9 @@ fsz_status fsz_compress_encode(const float* d_in, fsz_dims dims, fsz_eb_mode mod
                                void* d_ws, uint64_t ws_bytes, fsz_stream stream);
 
 /* Decompress one stream (Sec. 3.1 "Decompression", steps d1-d5) into d_out.
- * out_capacity_elems also bounds the workspace needed (fsz_workspace_bytes of it). */
+ * out_capacity_elems also bounds the workspace needed (fsz_workspace_bytes of it). A stream
+ * refused for its preamble leaves d_out as it was; one whose rate headers or means turn out
+ * malformed (FSZ_ERR_CORRUPT) may have had other chunks written. */
 fsz_status fsz_decompress(const void* d_in, uint64_t in_bytes, float* d_out,
                           uint64_t out_capacity_elems, void* d_ws, uint64_t ws_bytes,
                           fsz_stream stream);
@@ -242,7 +245,8 @@ fsz_status fsz_quality_stats(const float* d_orig, const float* d_recon, uint64_t
 fsz_status fsz_compress_batched(const fsz_cfield* d_fields, uint32_t nfields, uint64_t n_total,
                                 void* d_ws, uint64_t ws_bytes, fsz_stream stream);
 
-/* Decompress nfields streams in one persistent launch (plus a planning kernel).
+/* Decompress nfields streams in one persistent launch (plus a planning kernel and one that
+ * sizes the chunks from the rate headers).
  * d_fields: DEVICE array of nfields fsz_dfield. n_total_capacity = sum of the fields'
  * out_capacity_elems (sizes the workspace). */
 fsz_status fsz_decompress_batched(const fsz_dfield* d_fields, uint32_t nfields,
