@@ -467,6 +467,31 @@ def run_serving(fsz, inputs, dev, nreq: int = 20000, seed: int = 4, linger_us: i
             "closed_loop_vs_per_request": closed["gbs"] / per_req_gbs, "loads": levels}
 
 
+JOB_KEYS = ("field", "rel", "cr", "psnr_db", "errors_over_bound", "max_err_over_eb", "compress_gbs",
+            "encode_kernel_hbm_gbs", "decompress_hbm_gbs", "stats_gbs",
+            "encode_kernel_hbm_gbs_l2flushed", "decompress_hbm_gbs_l2flushed")
+
+
+def printed_line(record):
+    """The record as printed: floats to 6 digits, and of the per-job, ablation, tile and tuning
+    tables what the figures are quoted from (all of it goes to --details). Whoever reads the
+    output keeps a few KB of it, and a line cut short cannot be parsed."""
+    def short(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return [short(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+    line = dict(record)
+    line["jobs"] = [{k: j[k] for k in JOB_KEYS} for j in record["jobs"]]
+    for key, dropped in (("ablation", ("cr", "single_vs_multipass")), ("tiles", ("rows",)),
+                         ("batched", ("tuning_ms",))):
+        if record.get(key):
+            line[key] = {k: v for k, v in record[key].items() if k not in dropped}
+    return short(line)
+
+
 def run_ablation(fsz, fields, rels, dev, shape):
     """Sec. 6.4 (Table 7) and Sec. 6.3 on the bench fields: the compression ratio at each
     ablation step (Base = LZ1 with independent blocks, +Cross = the state carried across
@@ -734,6 +759,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="fsz", choices=["fsz", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--details", metavar="FILE", help="also write the whole record (every table) there")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-batched", action="store_true",
                     help="skip the 512-field batched vs per-field comparison")
@@ -1098,7 +1124,10 @@ def main():
                 "batched": batched,
                 "serving": serving,
                 "max_abs_err_last_job": p_last}
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(printed_line(line)))
     barrier(world)
     return 0
 
